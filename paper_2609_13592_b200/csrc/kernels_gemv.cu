@@ -1976,9 +1976,8 @@ int boosth::gemv_chain_launch(const boost_gemv_call_t* calls, uint32_t n_calls, 
 
 // A plain product on its own goes to the cluster kernel (kernels_pair.cu): one launch instead of the
 // product and its combine, no partial sums in memory.  Not where
-//   - a threadblock would sum more than kPairMaxDepth columns in one accumulator: the tensor cores' fp32
-//     adder truncates (about n 2^-24 of the result after n additions of 16 columns), and up to this
-//     depth the sums are as good as those of the shorter segments of the kernels above;
+//   - a threadblock's share of the columns would be more than kPairMaxDepth: longer rows on their own
+//     are not measured on it (in a step they are: the down product's 7168);
 //   - the rows are short: a threadblock's time is then its epilogue, and the kernels above finish
 //     tiles from tensor memory;
 //   - one of the process-wide switches that choose among the kernels above is not at its default.

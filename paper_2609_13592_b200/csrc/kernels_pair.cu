@@ -65,6 +65,7 @@ struct PairPhase {
   uint32_t split;            // 2: the cluster's threadblocks take half of K each; 1: every threadblock has rows of its own
   uint32_t image;            // units of an image: 16, or 8 where no worker has more (then a stage holds two k blocks)
   uint32_t max_images;       // images of the widest worker
+  uint32_t part_blocks;      // k blocks of an accumulator; 0: a quarter of a block
   void* y;
   int y_dtype;
   const __nv_bfloat16* residual;
@@ -89,19 +90,28 @@ struct PairParams {
 };
 
 // kN: the batch class of an instantiation (8, 16, 32, 64, 128, 256 rows).
-// Images that share an activation tile: from 128 rows on the tiles are the larger part of what an
-// SM draws from L2, so two images meet each (3-layer step, two against one: batch 128 1153 / 1150 us,
-// 200 1087 / 1110, 250 1236 / 1243: nearly even, since one image's epilogue then hides behind the next).
-__host__ __device__ constexpr uint32_t images_per_pass(uint32_t n) { return n >= 128 ? 2 : 1; }
-// Accumulator columns of a pass (an M = 128 product has at least 16), and how many passes tensor memory holds.
-__host__ __device__ constexpr uint32_t acc_cols(uint32_t n) { return (n < 16 ? 16 : n) * images_per_pass(n); }
-__host__ __device__ constexpr uint32_t acc_bufs(uint32_t n) { return acc_cols(n) > 256 ? 1 : 2; }
-__host__ __device__ constexpr uint32_t tmem_cols(uint32_t n) { return acc_bufs(n) * acc_cols(n) < 32 ? 32 : acc_bufs(n) * acc_cols(n); }
 // Activations by tiled TMA copies, or by one warp's 16-byte copies (3-layer step, 16-byte copies against
 // TMA: batch 1 465 / 473 us, 8 500 / 506, 32 636 / 641; more rows are too many copies for one warp).
 __host__ __device__ constexpr bool x_by_tma(uint32_t n) { return n > 32; }
-// k blocks of an activation slot
-__host__ __device__ constexpr uint32_t x_blocks(uint32_t n) { return n >= 128 ? 1 : 2; }
+// k blocks of an activation slot.  (Up to 16 rows four: half the barrier polls and commits of the MMA warp.)
+__host__ __device__ constexpr uint32_t x_blocks(uint32_t n) { return n <= 16 ? 4 : n >= 128 ? 1 : 2; }
+// The tensor cores' fp32 adder truncates: every MMA that adds to an accumulator takes about 2.7e-8 of
+// what it holds, always towards zero, so a sum over n MMAs is off by n / 2 times that (2-norm against
+// fp64, normal inputs, 32 / 128 / 256 MMAs: 4.5e-7, 2.1e-6, 4.4e-6).  An accumulator therefore holds a PART
+// of the columns only (PairPhase::part_blocks), and the epilogue warps take the parts out of tensor
+// memory as they come and add them up where additions round to nearest.
+// Parts of part_cols columns (an M = 128 product has at least 16) change hands in slots of up to
+// slot_parts; as many slots as tensor memory holds are in flight.
+__host__ __device__ constexpr uint32_t part_cols(uint32_t n) { return n < 16 ? 16 : n; }
+__host__ __device__ constexpr uint32_t slot_parts(uint32_t n) { return n <= 8 ? 16 : n <= 16 ? 4 : n <= 64 ? 2 : 1; }
+__host__ __device__ constexpr uint32_t slot_cols(uint32_t n) { return part_cols(n) * slot_parts(n); }
+constexpr uint32_t kMaxAccSlots = 8;
+__host__ __device__ constexpr uint32_t acc_slots(uint32_t n) { return 512 / slot_cols(n) < kMaxAccSlots ? 512 / slot_cols(n) : kMaxAccSlots; }
+__host__ __device__ constexpr uint32_t tmem_cols(uint32_t n) { return acc_slots(n) * slot_cols(n); }
+// k blocks of a slot whose parts are part_blocks (0: a quarter of a block, one MMA) each.
+__host__ __device__ constexpr uint32_t slot_blocks(uint32_t n, uint32_t part_blocks) {
+  return part_blocks == 0 ? slot_parts(n) / 4 : part_blocks == 1 ? slot_parts(n) : part_blocks;
+}
 // Epilogue warps: a short product's last accumulator is finished by all of them at the end of a phase,
 // which at large batches is bound by their instruction latency.
 __host__ __device__ constexpr uint32_t epi_warps(uint32_t n) { return n <= 32 ? 8 : 16; }
@@ -115,6 +125,9 @@ __host__ __device__ constexpr uint32_t chunk_cols(uint32_t n) { return n < 64 ? 
 // (up to 32 rows) or in the activation slots, which are idle then.
 __host__ __device__ constexpr uint32_t rounds_of(uint32_t n) { return n >= 256 ? 2 : 1; }
 __host__ __device__ constexpr uint32_t sums_bytes(uint32_t n) { return chunk_cols(n) * kRowTile * 4; }
+
+template <auto kValue>
+struct Const { static constexpr auto value = kValue; };
 
 // Rows [u0, u1) (in units) of worker w of W.
 __host__ __device__ inline void worker_range(uint32_t n_units, uint32_t w, uint32_t W, uint32_t& u0, uint32_t& u1) {
@@ -152,24 +165,67 @@ __device__ __forceinline__ void umma_low(uint32_t d_tmem, uint32_t a_low, uint32
       "r"(a_low), "r"(b_low), "r"(idesc), "r"(accumulate), "n"(kDescHigh)
       : "memory");
 }
-// kC consecutive columns of this warp's 32 tensor-memory lanes.
-template <uint32_t kC>
-__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, float (&v)[kC]) {
-  static_assert(kC == 2 || kC == 4 || kC == 8, "2, 4 or 8 columns");
-  uint32_t r[kC];
-  if constexpr (kC == 2)
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(taddr) : "memory");
-  else if constexpr (kC == 4)
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
-  else
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr)
-                 : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (uint32_t i = 0; i < kC; ++i) v[i] = __uint_as_float(r[i]);
+// Columns of this warp's 32 tensor-memory lanes, with the wait for them in the same statement, so that
+// nothing is done with the registers before it: 8 at one address, 4, 8 at each of two, 2 at each of eight.
+__device__ __forceinline__ void tmem_ld_8(uint32_t addr, float (&v)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+      : "r"(addr)
+      : "memory");
 }
+__device__ __forceinline__ void tmem_ld_4(uint32_t addr, float (&v)[4]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+      : "r"(addr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld_2x8(uint32_t addr0, uint32_t addr1, float (&v)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%16];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%17];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=&f"(v[0]), "=&f"(v[1]), "=&f"(v[2]), "=&f"(v[3]), "=&f"(v[4]), "=&f"(v[5]), "=&f"(v[6]), "=&f"(v[7]), "=&f"(v[8]), "=&f"(v[9]),
+        "=&f"(v[10]), "=&f"(v[11]), "=&f"(v[12]), "=&f"(v[13]), "=&f"(v[14]), "=&f"(v[15])
+      : "r"(addr0), "r"(addr1)
+      : "memory");
+}
+template <uint32_t kStep>
+__device__ __forceinline__ void tmem_ld_8x2(uint32_t addr, float (&v)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%16];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%2,%3}, [%17];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%4,%5}, [%18];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%6,%7}, [%19];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%8,%9}, [%20];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%10,%11}, [%21];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%12,%13}, [%22];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%14,%15}, [%23];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=&f"(v[0]), "=&f"(v[1]), "=&f"(v[2]), "=&f"(v[3]), "=&f"(v[4]), "=&f"(v[5]), "=&f"(v[6]), "=&f"(v[7]), "=&f"(v[8]), "=&f"(v[9]),
+        "=&f"(v[10]), "=&f"(v[11]), "=&f"(v[12]), "=&f"(v[13]), "=&f"(v[14]), "=&f"(v[15])
+      : "r"(addr), "r"(addr + kStep), "r"(addr + 2 * kStep), "r"(addr + 3 * kStep), "r"(addr + 4 * kStep), "r"(addr + 5 * kStep),
+        "r"(addr + 6 * kStep), "r"(addr + 7 * kStep)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st_8(uint32_t addr, const float* v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0,%1,%2,%3,%4,%5,%6,%7};" ::"f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]),
+               "f"(v[5]), "f"(v[6]), "f"(v[7]), "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// Two fp32 additions (round to nearest) in one instruction.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tadd.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return add2(a, make_float2(-b.x, -b.y)); }
 __device__ __forceinline__ float bf16_round(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
 
 // Barrier operations and copies on shared-memory addresses (the loops below step through them).
@@ -240,11 +296,11 @@ __device__ __noinline__ uint32_t host_bytes_of_range(const PairPhase& q, uint32_
 
 template <uint32_t kN>
 __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairParams p) {
-  constexpr uint32_t kAcc = acc_cols(kN), kBufs = acc_bufs(kN), kIpp = images_per_pass(kN), kXB = x_blocks(kN);
+  constexpr uint32_t kXB = x_blocks(kN), kSlots = acc_slots(kN), kSlotCols = slot_cols(kN);
   constexpr bool kTmaX = x_by_tma(kN);
   constexpr uint32_t kEpiWarps = epi_warps(kN), kEpiThreads = kEpiWarps * 32;
   constexpr bool kBig = kN >= 64;
-  constexpr uint32_t CW = chunk_cols(kN), CH = kBig ? 8 : kN / 4, HG = kEpiWarps / 4;   // columns of a chunk; of one tensor-memory load; warps that share lanes
+  constexpr uint32_t CW = chunk_cols(kN), CH = kBig ? 8 : kN / 2, HG = kEpiWarps / 4;   // columns of a chunk; of a group; warps that share lanes
   extern __shared__ uint8_t smem_raw[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t n_stages = p.n_stages, x_slots = p.x_slots;
@@ -254,7 +310,7 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
   // (an 8-row activation tile is read as 16 rows: 1 KiB behind the slots)
   float* sums = reinterpret_cast<float*>(x_ring + x_slot * x_slots + 1024u);
   __shared__ uint64_t w_full[kMaxStages], w_empty[kMaxStages], x_full[kMaxXSlots], x_empty[kMaxXSlots];
-  __shared__ uint64_t acc_full[2], acc_empty[2], xch_full, xch_free, go, drained;
+  __shared__ uint64_t acc_full[kMaxAccSlots], acc_empty[kMaxAccSlots], xch_full, xch_free, go, drained;
   __shared__ uint32_t s_tmem;
   __shared__ uint32_t s_rec[kMaxPhases];
   __shared__ float s_rs[kN], s_red[kEpiThreads];
@@ -272,7 +328,7 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
   if (tid == 0) {
     for (uint32_t s = 0; s < n_stages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); }
     for (uint32_t s = 0; s < x_slots; ++s) { mbar_init(&x_full[s], kTmaX ? 1 : 32); mbar_init(&x_empty[s], 1); }
-    for (uint32_t s = 0; s < 2; ++s) {
+    for (uint32_t s = 0; s < kSlots; ++s) {
       mbar_init(&acc_full[s], 1);
       mbar_init(&acc_empty[s], kEpiWarps);
     }
@@ -320,8 +376,8 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
     uint32_t stage = 0, parity = 1;
     bool my_turn = warp == 0;
     // Per stage: wait, announce the bytes, copy.  Everything else is kept out of the loop: the lanes
-    // hold the pieces' addresses (part of the run x lower / upper rows; x image of the pass, or x k
-    // block of an image of 8), and step through K on their own.
+    // hold the pieces' addresses (part of the run x lower / upper rows; x k block of an image of 8), and
+    // step through K on their own.
     auto produce = [&](const PairPhase& q, uint32_t ph) -> bool {
       const Part w = part_of(q);
       const uint32_t image = q.image, k_blocks = q.k_blocks, n_pages = q.n_pages;
@@ -336,13 +392,12 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
       __syncwarp();
       const uint32_t step = twos ? 2u : 1u;
       const uint32_t sub = lane >> 2, part = (lane >> 1) & 1u, half = lane & 1u;
-      for (uint32_t pa = w.u0; pa < w.u1; pa += w.run * kIpp) {
-        const uint32_t images = min(kIpp, (w.u1 - pa + w.run - 1) / w.run);
-        // this lane's piece: units [a, b) of an image's run (its part before or behind the wrap), lower or upper rows, k block kb + second
-        const uint32_t second = twos ? sub & 1u : 0u, img = twos ? 0u : min(sub, images - 1);
-        const uint32_t ua = pa + img * w.run, ub = min(w.u1, ua + w.run), mid = min(ub, (ua / image + 1) * image);
+      for (uint32_t ua = w.u0; ua < w.u1; ua += w.run) {
+        // this lane's piece: units [a, b) of the image's run (its part before or behind the wrap), lower or upper rows, k block kb + second
+        const uint32_t second = twos ? sub & 1u : 0u;
+        const uint32_t ub = min(w.u1, ua + w.run), mid = min(ub, (ua / image + 1) * image);
         const uint32_t a = part ? mid : ua, b = part ? ub : mid;
-        bool mine = sub < (twos ? 2u : images) && a < b;
+        bool mine = sub < step && a < b;
         uint32_t bytes = (b - a) * 512u;
         if (mine && b - a == kUnitsPerTile) {   // a whole row tile is one copy
           bytes = kBlockBytes;
@@ -360,24 +415,22 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
           src = base + (size_t)(blk % kBlocksPerPage) * kBlockBytes + in_block;
         };
         if (mine && w.kb0 + second < w.kb1) locate();
-        const uint32_t last_tx = (min(w.u1, pa + w.run * images) - (pa + w.run * (images - 1))) * 1024u;
+        const uint32_t tx = (ub - ua) * 1024u * step;
         for (uint32_t kb = w.kb0; kb < w.kb1; kb += step) {
           if (mine && second && kb + 1 == w.kb1) {
             // an odd last block is its own partner (it meets zeros, or nothing)
             const uint32_t b0 = blk - 1;
             src = static_cast<const uint8_t*>(page_ptr[b0 / kBlocksPerPage]) + (size_t)(b0 % kBlocksPerPage) * kBlockBytes + in_block;
           }
-          for (uint32_t i = 0; i < images; ++i) {
-            if (my_turn) {
-              if (!wait(empty_a + stage * 8, parity)) return false;
-              const uint32_t full = full_a + stage * 8;
-              if (lane == 0) expect_tx(full, (i + 1 == images ? last_tx : w.run * 1024u) * step);
-              __syncwarp();
-              if (mine && img == i) bulk_copy(to + stage * kStageBytes, src, bytes, full);
-            }
-            my_turn = !my_turn;
-            if (++stage == n_stages) { stage = 0; parity ^= 1u; }
+          if (my_turn) {
+            if (!wait(empty_a + stage * 8, parity)) return false;
+            const uint32_t full = full_a + stage * 8;
+            if (lane == 0) expect_tx(full, tx);
+            __syncwarp();
+            if (mine) bulk_copy(to + stage * kStageBytes, src, bytes, full);
           }
+          my_turn = !my_turn;
+          if (++stage == n_stages) { stage = 0; parity ^= 1u; }
           blk += step;
           src += step * kBlockBytes;
           if (mine && blk % kBlocksPerPage < step && kb + step + second < w.kb1) locate();
@@ -403,7 +456,7 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
     uint32_t xs = 0, parity = 1;
     auto produce = [&](const PairPhase& q, uint32_t ph) -> bool {
       const Part w = part_of(q);
-      const uint32_t K = q.K, run = w.run * kIpp;
+      const uint32_t K = q.K, run = w.run;
       if constexpr (kTmaX) {
         fence_proxy_async_all();   // x was written with ordinary stores and is read through the TMA unit
         for (uint32_t pa = w.u0; pa < w.u1; pa += run)
@@ -424,23 +477,27 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
         const uint32_t to0 = x_a + r0 * 128u + ((c ^ r0) << 4), to1 = x_a + (r0 + 4) * 128u + ((c ^ (r0 + 4)) << 4);   // rows 8 i + r0, 8 i + 4 + r0
         const __nv_bfloat16* const x0 = q.x + (size_t)r0 * K + (c * 8u < K ? c * 8u : 0u);
         for (uint32_t pa = w.u0; pa < w.u1; pa += run)
-          for (uint32_t kb = w.kb0; kb < w.kb1; kb += 2) {
+          for (uint32_t kb = w.kb0; kb < w.kb1; kb += kXB) {
             if (!wait(empty_a + xs * 8, parity)) return false;
-            const uint32_t k0 = kb * 64u + c * 8u;
-            const bool in0 = k0 < K, in1 = k0 + 64u < K && kb + 1 < w.kb1;   // (behind an odd last block: zeros)
-            const uint32_t n0 = in0 ? 16u : 0u, n1 = in1 ? 16u : 0u;
-            const uint32_t d1 = in1 ? 64u : 0u, at = xs * x_slot;
-            const __nv_bfloat16* src = x0 + (in0 ? kb * 64u : 0u);
+            const uint32_t at = xs * x_slot;
+            uint32_t n[kXB], off[kXB];   // bytes and columns; behind the last block, and behind the last column in it, zeros
+#pragma unroll
+            for (uint32_t b = 0; b < kXB; ++b) {
+              const bool in = kb + b < w.kb1 && (kb + b) * 64u + c * 8u < K;
+              n[b] = in ? 16u : 0u;
+              off[b] = in ? b * 64u : 0u;
+            }
+            const __nv_bfloat16* src = x0 + (n[0] ? kb * 64u : 0u);
 #pragma unroll
             for (uint32_t i = 0; i < kN / 8; ++i) {
               if (i * 8 + r0 < M_b) {
-                cp_async_16s(to0 + at + i * 1024u, src, n0);
-                cp_async_16s(to0 + at + i * 1024u + x_block, src + d1, n1);
+#pragma unroll
+                for (uint32_t b = 0; b < kXB; ++b) cp_async_16s(to0 + at + i * 1024u + b * x_block, src + off[b], n[b]);
               }
               src += (size_t)4 * K;
               if (i * 8 + 4 + r0 < M_b) {
-                cp_async_16s(to1 + at + i * 1024u, src, n0);
-                cp_async_16s(to1 + at + i * 1024u + x_block, src + d1, n1);
+#pragma unroll
+                for (uint32_t b = 0; b < kXB; ++b) cp_async_16s(to1 + at + i * 1024u + b * x_block, src + off[b], n[b]);
               }
               src += (size_t)4 * K;
             }
@@ -481,9 +538,11 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
     const uint32_t idesc64 = umma_idesc_bf16_f32(kRowTile / 2, nb);
     const uint32_t full_a = smem_u32(w_full), empty_a = smem_u32(w_empty), xfull_a = smem_u32(x_full), xempty_a = smem_u32(x_empty);
     const uint32_t w_low = desc_low(smem_u32(ring)), x_low = desc_low(smem_u32(x_ring)), x_step = x_slot / 16, x_half = x_block / 16;
-    uint32_t stage = 0, parity = 0, xs = 0, xpar = 0, acc = 0;
+    const uint32_t afull_a = smem_u32(acc_full), aempty_a = smem_u32(acc_empty);
+    uint32_t stage = 0, parity = 0, xs = 0, xpar = 0, as = 0, apar = 1;
     auto next_stage = [&]() { if (++stage == n_stages) { stage = 0; parity ^= 1u; } };
     auto next_slot = [&]() { if (++xs == x_slots) { xs = 0; xpar ^= 1u; } };
+    auto next_acc = [&]() { if (++as == kSlots) { as = 0; apar ^= 1u; } };
     // odd lanes poll one barrier, even lanes the other
     auto wait_two = [&](uint32_t bar0, uint32_t par0, uint32_t bar1, uint32_t par1) -> bool {
       const uint32_t bar = (lane & 1u) ? bar1 : bar0, par = (lane & 1u) ? par1 : par0;
@@ -493,39 +552,113 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
       return __all_sync(0xFFFFFFFFu, ok) != 0;
     };
     auto wait_one = [&](uint32_t bar, uint32_t par) -> bool { return wait_two(bar, par, bar, par); };
-    // One k block: 4 MMAs.  (16 columns on: 32 bytes, 2 in a descriptor's address field, which counts in 16 bytes)
-    auto mma_block = [&](uint32_t d, uint32_t wl, uint32_t xl, uint32_t id, uint32_t accumulate) {
-#pragma unroll
-      for (uint32_t ks = 0; ks < 4; ++ks) umma_low(d, wl + 2 * ks, xl + 2 * ks, id, ks ? 1u : accumulate);
+    auto wait_three = [&](uint32_t bar0, uint32_t par0, uint32_t bar1, uint32_t par1, uint32_t bar2, uint32_t par2) -> bool {
+      return wait_two(bar0, par0, (lane & 2u) ? bar2 : bar1, (lane & 2u) ? par2 : par1);
     };
-    auto multiply = [&](const PairPhase& q) -> bool {
+    // image8: images of 8 units (two k blocks a stage).  mode: parts of a quarter of a k block (0), a k block (1), several (2).
+    // (Compile-time, and slots around the loop over stages, for this warp's instruction latency: with one
+    // loop that decides at run time a step of one sequence took 4230 us instead of 3570, all else equal.)
+    auto multiply = [&](const PairPhase& q, auto image8, auto mode) -> bool {
+      constexpr bool kImage8 = decltype(image8)::value;
+      constexpr uint32_t kMode = decltype(mode)::value;
       const Part w = part_of(q);
-      const uint32_t image = q.image;
-      for (uint32_t pa = w.u0; pa < w.u1; pa += w.run * kIpp, ++acc) {
-        const uint32_t buf = acc % kBufs, d = tmem + buf * kAcc;
-        if (!wait_one(smem_u32(&acc_empty[buf]), ((acc / kBufs) & 1u) ^ 1u)) return false;
-        uint32_t accumulate = 0;
-        if (image == 8) {
-          for (uint32_t kb = w.kb0; kb < w.kb1; kb += 2) {
-            const uint32_t wl = w_low + stage * (kStageBytes / 16), xl = x_low + xs * x_step;
-            const uint32_t free_w = empty_a + stage * 8, free_x = xempty_a + xs * 8;
-            if (!wait_two(full_a + stage * 8, parity, xfull_a + xs * 8, xpar)) return false;
-            if constexpr (!kTmaX) fence_proxy_async_smem();   // (activations that came through the load/store path)
-            tc_fence_after_sync();
-            next_stage();
-            next_slot();
-            if constexpr (kXB == 2) {
-              if (elect_one()) {
-                mma_block(d, wl, xl, idesc64, accumulate);
-                if (kb + 1 < w.kb1) mma_block(d, wl + kStageBytes / 32, xl + x_half, idesc64, 1u);
-                commit(free_w);
-                commit(free_x);
+      const uint32_t slot_n = slot_blocks(kN, kMode == 2 ? q.part_blocks : kMode), id = kImage8 ? idesc64 : idesc;
+      constexpr uint32_t kBlockCols = kMode == 2 ? 0 : kMode == 1 ? part_cols(kN) : 4 * part_cols(kN), kNext = kMode == 0 ? part_cols(kN) : 0;
+      // One k block: 4 MMAs.  (16 columns on: 32 bytes, 2 in a descriptor's address field, which counts in 16 bytes)
+      auto mma_block = [&](uint32_t d, uint32_t wl, uint32_t xl, uint32_t accumulate) {
+#pragma unroll
+        for (uint32_t ks = 0; ks < 4; ++ks)
+          umma_low(d + ks * kNext, wl + 2 * ks, xl + 2 * ks, id, kMode == 0 ? 0u : ks == 0 ? accumulate : 1u);
+      };
+      for (uint32_t ua = w.u0; ua < w.u1; ua += w.run) {
+        for (uint32_t kb = w.kb0; kb < w.kb1;) {   // a slot of accumulators: the epilogue warps have read what was there
+          const uint32_t kb_end = min(kb + slot_n, w.kb1), done = afull_a + as * 8;
+          [[maybe_unused]] const uint32_t kb_first = kb;
+          uint32_t d = tmem + as * kSlotCols, accumulate = 0;
+          if constexpr (kMode != 0)
+            if (!wait_one(aempty_a + as * 8, apar)) return false;
+          if constexpr (kXB == 4) {
+            constexpr uint32_t kPer = kImage8 ? 2 : 1;   // k blocks of a stage
+            for (; kb < kb_end; kb += kXB) {
+              const uint32_t n = min(kXB, kb_end - kb), xl = x_low + xs * x_step, free_x = xempty_a + xs * 8;
+#pragma unroll
+              for (uint32_t j = 0; j < kXB; j += kPer) {
+                if (j && j >= n) break;
+                const uint32_t wl = w_low + stage * (kStageBytes / 16), full_w = full_a + stage * 8, free_w = empty_a + stage * 8;
+                const bool last = j + kPer >= n;
+                bool ok;
+                if (j) ok = wait_one(full_w, parity);
+                else if (kMode == 0 && kb == kb_first) ok = wait_three(full_w, parity, xfull_a + xs * 8, xpar, aempty_a + as * 8, apar);
+                else ok = wait_two(full_w, parity, xfull_a + xs * 8, xpar);
+                if (!ok) return false;
+                if (j == 0) fence_proxy_async_smem();   // (activations that came through the load/store path)
+                tc_fence_after_sync();
+                next_stage();
+                if (elect_one()) {
+                  mma_block(d + j * kBlockCols, wl, xl + j * x_half, j ? kMode == 2 : accumulate);
+                  if (kImage8 && j + 1 < n) mma_block(d + (j + 1) * kBlockCols, wl + kStageBytes / 32, xl + (j + 1) * x_half, kMode == 2);
+                  commit(free_w);
+                  if (last) commit(free_x);
+                  if (kMode == 0 && last && kb + kXB >= kb_end) commit(done);
+                }
+                __syncwarp();
               }
-            } else {
-              // the activation tiles of the two k blocks are slots of their own
+              next_slot();
+              d += kXB * kBlockCols;
+              accumulate = kMode == 2;
+            }
+            kb = kb_end;
+          } else if constexpr (kXB == 2) {
+            for (; kb < kb_end; kb += 2) {
+              const uint32_t wl = w_low + stage * (kStageBytes / 16), xl = x_low + xs * x_step;
+              const uint32_t free0 = empty_a + stage * 8, free_x = xempty_a + xs * 8;
+              if (!wait_two(full_a + stage * 8, parity, xfull_a + xs * 8, xpar)) return false;
+              if constexpr (!kTmaX) fence_proxy_async_smem();
+              tc_fence_after_sync();
+              next_stage();
+              next_slot();
+              if constexpr (kImage8) {
+                if (elect_one()) {
+                  mma_block(d, wl, xl, accumulate);
+                  if (kb + 1 < w.kb1) mma_block(d + kBlockCols, wl + kStageBytes / 32, xl + x_half, kMode == 2);
+                  commit(free0);
+                  commit(free_x);
+                }
+              } else {
+                const bool both = kb + 1 < w.kb1;
+                if (elect_one()) {
+                  mma_block(d, wl, xl, accumulate);
+                  commit(free0);
+                  if (!both) commit(free_x);
+                }
+                __syncwarp();
+                if (both) {
+                  const uint32_t wl1 = w_low + stage * (kStageBytes / 16), free1 = empty_a + stage * 8;
+                  if (!wait_one(full_a + stage * 8, parity)) return false;
+                  tc_fence_after_sync();
+                  next_stage();
+                  if (elect_one()) {
+                    mma_block(d + kBlockCols, wl1, xl + x_half, kMode == 2);
+                    commit(free1);
+                    commit(free_x);
+                  }
+                }
+              }
+              __syncwarp();
+              d += 2 * kBlockCols;
+              accumulate = kMode == 2;
+            }
+          } else if constexpr (kImage8 && kMode == 2) {
+            for (; kb < kb_end; kb += 2) {   // (the activation tiles of a stage's two k blocks are slots of their own)
               const bool both = kb + 1 < w.kb1;
+              const uint32_t wl = w_low + stage * (kStageBytes / 16), xl = x_low + xs * x_step;
+              const uint32_t free_w = empty_a + stage * 8, free_x = xempty_a + xs * 8;
+              if (!wait_two(full_a + stage * 8, parity, xfull_a + xs * 8, xpar)) return false;
+              tc_fence_after_sync();
+              next_stage();
+              next_slot();
               if (elect_one()) {
-                mma_block(d, wl, xl, idesc64, accumulate);
+                mma_block(d, wl, xl, accumulate);
                 commit(free_x);
                 if (!both) commit(free_w);
               }
@@ -536,83 +669,50 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
                 tc_fence_after_sync();
                 next_slot();
                 if (elect_one()) {
-                  mma_block(d, wl + kStageBytes / 32, xl1, idesc64, 1u);
+                  mma_block(d, wl + kStageBytes / 32, xl1, 1u);
                   commit(free_x1);
                   commit(free_w);
                 }
+                __syncwarp();
               }
+              accumulate = 1;
             }
-            __syncwarp();
-            accumulate = 1;
-          }
-        } else if constexpr (kXB == 2) {
-          for (uint32_t kb = w.kb0; kb < w.kb1; kb += 2) {
-            const bool both = kb + 1 < w.kb1;
-            const uint32_t wl = w_low + stage * (kStageBytes / 16), xl = x_low + xs * x_step;
-            const uint32_t free0 = empty_a + stage * 8, free_x = xempty_a + xs * 8;
-            if (!wait_two(full_a + stage * 8, parity, xfull_a + xs * 8, xpar)) return false;
-            if constexpr (!kTmaX) fence_proxy_async_smem();
-            tc_fence_after_sync();
-            next_stage();
-            next_slot();
-            if (elect_one()) {
-              mma_block(d, wl, xl, idesc, accumulate);
-              commit(free0);
-              if (!both) commit(free_x);
-            }
-            __syncwarp();
-            if (both) {
-              const uint32_t wl1 = w_low + stage * (kStageBytes / 16), free1 = empty_a + stage * 8;
-              if (!wait_one(full_a + stage * 8, parity)) return false;
+          } else {
+            for (; kb < kb_end; ++kb) {   // (a part is a k block: an image of 8 may leave a slot in the middle of a stage)
+              const bool second = kImage8 && ((kb - w.kb0) & 1u), last = !kImage8 || second || kb + 1 == w.kb1;
+              const uint32_t wl = w_low + stage * (kStageBytes / 16) + (second ? kStageBytes / 32 : 0u), xl = x_low + xs * x_step;
+              const uint32_t free_w = empty_a + stage * 8, free_x = xempty_a + xs * 8;
+              if (!wait_two(full_a + stage * 8, parity, xfull_a + xs * 8, xpar)) return false;
               tc_fence_after_sync();
-              next_stage();
+              if (last) next_stage();
+              next_slot();
               if (elect_one()) {
-                mma_block(d, wl1, xl + x_half, idesc, 1u);
-                commit(free1);
+                mma_block(d, wl, xl, accumulate);
                 commit(free_x);
+                if (last) commit(free_w);
               }
               __syncwarp();
+              d += kBlockCols;
+              accumulate = kMode == 2;
             }
-            accumulate = 1;
           }
-        } else {
-          const uint32_t images = min(kIpp, (w.u1 - pa + w.run - 1) / w.run);
-          for (uint32_t kb = w.kb0; kb < w.kb1; ++kb) {   // the images of the pass meet one activation tile
-            const uint32_t xl = x_low + xs * x_step, free_x = xempty_a + xs * 8;
-            uint32_t wl = w_low + stage * (kStageBytes / 16), free_w = empty_a + stage * 8;
-            if (!wait_two(full_a + stage * 8, parity, xfull_a + xs * 8, xpar)) return false;
-            tc_fence_after_sync();
-            next_stage();
-            next_slot();
-            if (elect_one()) {
-              mma_block(d, wl, xl, idesc, accumulate);
-              commit(free_w);
-              if (images == 1) commit(free_x);
-            }
+          if constexpr (kMode != 0) {
+            if (elect_one()) commit(done);
             __syncwarp();
-            if (images == 2) {
-              wl = w_low + stage * (kStageBytes / 16);
-              free_w = empty_a + stage * 8;
-              if (!wait_one(full_a + stage * 8, parity)) return false;
-              tc_fence_after_sync();
-              next_stage();
-              if (elect_one()) {
-                mma_block(d + kN, wl, xl, idesc, accumulate);
-                commit(free_w);
-                commit(free_x);
-              }
-              __syncwarp();
-            }
-            accumulate = 1;
           }
+          next_acc();
         }
-        if (elect_one()) commit(smem_u32(&acc_full[buf]));
-        __syncwarp();
       }
       return true;
     };
+    auto multiply_phase = [&](const PairPhase& q) -> bool {
+      auto with_mode = [&](auto mode) { return q.image == 8 ? multiply(q, Const<true>(), mode) : multiply(q, Const<false>(), mode); };
+      if constexpr (kN == 8)
+        if (q.part_blocks == 0) return with_mode(Const<0u>());
+      return q.part_blocks == 1 ? with_mode(Const<1u>()) : with_mode(Const<2u>());
+    };
     for (uint32_t ph = 0; ph < p.n_phases; ++ph)
-      if (!multiply(p.ph[ph])) break;
+      if (!multiply_phase(p.ph[ph])) break;
     if (s_abort) {
       // nothing may be in the tensor cores' pipeline when its operands and accumulators go away
       if (elect_one()) commit(smem_u32(&drained));
@@ -621,13 +721,14 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
     }
   } else if (warp >= kEpiWarp0) {
     // ------------------------------------------------------------------ epilogue
-    // An image's sums go from tensor memory to shared memory (half of the columns to the peer's where
-    // two threadblocks share the rows), and from there to all epilogue threads, which finish a pair of
-    // rows 64 apart (gate / up, the two halves of a rotary pair) for a few sequences each.
+    // An image's accumulators are added up as they come, and the sums go to shared memory (half of the
+    // columns to the peer's where two threadblocks share the rows), and from there to all epilogue
+    // threads, which finish a pair of rows 64 apart (gate / up, the two halves of a rotary pair) for a
+    // few sequences each.
     const uint32_t et = tid - kEpiWarp0 * 32, quarter = warp & 3u, hh = (warp - kEpiWarp0) >> 2;
     const uint32_t l128 = quarter * 32u + lane;   // tensor-memory lane
     const uint32_t skip = et == 0 ? skip_arrivals_of(p.ws) : 0u;
-    uint32_t acc = 0, n_xch = 0;
+    uint32_t as = 0, apar = 0, n_xch = 0;
     pdl_wait();
     for (uint32_t ph = 0; ph < p.n_phases; ++ph) {
       const PairPhase& q = p.ph[ph];
@@ -816,102 +917,241 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
       // The accumulator row of this lane.  Of an M = 64 product, 16 rows lie in the first 16 lanes of every 32.
       const bool m64 = image == 8, holds = !m64 || lane < 16;
       const uint32_t row = m64 ? quarter * 16u + lane : l128;
-      // Columns [c0, c0 + cols) of the accumulator at `from`, to a buffer of shared memory.
-      auto drain = [&](uint32_t from, uint32_t c0, uint32_t cols, float* to) {   // (a warp together: the load is collective)
-        for (uint32_t c = hh * CH; c < cols; c += HG * CH) {
-          float v[CH];
-          tmem_ld_cols<CH>(from + c0 + c, v);
-#pragma unroll
-          for (uint32_t j = 0; j < CH; ++j)
-            if (holds) to[(c + j) * kRowTile + row] = v[j];
-        }
-      };
-      auto release_acc = [&](uint32_t buf) {
+      // The sums of an image: group i is the CH columns from column(i) on.
+      constexpr uint32_t kGroups = kN / (HG * CH);
+      auto column = [&](uint32_t i) { return hh * CH + i * (HG * CH); };
+      const uint32_t lane_base = tmem + ((quarter * 32u) << 16);
+      const uint32_t part_blocks = q.part_blocks, slot_n = slot_blocks(kN, part_blocks);
+      // From 128 rows on the sums would be up to half of a thread's registers: they stay in tensor memory, in
+      // the slot of the last part added, which is given back when the epilogue has read them.  (Registers:
+      // 244 - 508 bytes of spills at 256 rows, 6-layer step at batch 250 2147 - 2350 us instead of 2045.)
+      constexpr bool kParkSums = kN >= 128;
+      float sum[kParkSums ? 1 : kGroups][CH];
+      uint32_t parked = 0;   // the slot kept
+      auto release_slot = [&](uint32_t slot) {
         tc_fence_before_sync();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&acc_empty[buf]);
+        if (lane == 0) mbar_arrive(&acc_empty[slot]);
       };
-      const uint32_t lane_base = tmem + ((quarter * 32u) << 16);
+      auto group_sums = [&](uint32_t i, float (&v)[CH]) {   // i: a constant, except where the sums are parked
+        if constexpr (kParkSums) {
+          tmem_ld_8(lane_base + parked * kSlotCols + column(i), v);
+        } else {
+#pragma unroll
+          for (uint32_t e = 0; e < CH; ++e) v[e] = sum[i][e];
+        }
+      };
+      // Every part of the image's columns, as its slot comes.  take(from, n): the n parts at tensor-memory address `from`.
+      auto each_slot = [&](auto take) {
+        for (uint32_t kb = w.kb0; kb < w.kb1; kb += slot_n) {
+          wait(smem_u32(&acc_full[as]), apar);
+          __syncwarp();
+          tc_fence_after_sync();
+          const uint32_t here = min(slot_n, w.kb1 - kb);
+          if (column(0) < M_b) take(lane_base + as * kSlotCols + column(0), part_blocks > 1 ? 1u : part_blocks ? here : 4 * here);
+          release_slot(as);
+          if (++as == kSlots) { as = 0; apar ^= 1u; }
+        }
+      };
+      auto add = [&](float* to, const float* v, uint32_t n) {
+#pragma unroll
+        for (uint32_t j = 0; j < n; j += 2) {
+          const float2 t = add2(make_float2(to[j], to[j + 1]), make_float2(v[j], v[j + 1]));
+          to[j] = t.x;
+          to[j + 1] = t.y;
+        }
+      };
+      auto accumulate = [&]() {
+        if constexpr (kParkSums) {
+          for (uint32_t kb = w.kb0; kb < w.kb1; kb += slot_n) {   // (a slot is one part)
+            wait(smem_u32(&acc_full[as]), apar);
+            __syncwarp();
+            tc_fence_after_sync();
+            if (kb != w.kb0) {   // the sum so far, from the slot before, goes on top of this part
+              const uint32_t before = lane_base + parked * kSlotCols, here = lane_base + as * kSlotCols;
+#pragma unroll
+              for (uint32_t i = 0; i < kGroups; ++i) {
+                if (column(i) >= M_b) continue;   // (columns beyond the batch: nobody's)
+                float v[16];
+                tmem_ld_2x8(before + column(i), here + column(i), v);
+                add(v, v + 8, 8);
+                tmem_st_8(here + column(i), v);
+              }
+              tmem_st_wait();
+              release_slot(parked);
+            }
+            parked = as;
+            if (++as == kSlots) { as = 0; apar ^= 1u; }
+          }
+        } else {
+#pragma unroll
+          for (uint32_t i = 0; i < kGroups; ++i)
+#pragma unroll
+            for (uint32_t j = 0; j < CH; ++j) sum[i][j] = 0.f;
+          if constexpr (kN == 8) {
+            if (part_blocks == 0) {
+              // batches of 1 and 2, whose sums compare with those of CUDA cores: four parts added up pairwise,
+              // then a compensated sum (Knuth's two-sum: t + error = s + p exactly)
+              float2 s = make_float2(0.f, 0.f), lost = s;
+              each_slot([&](uint32_t from, uint32_t n_parts) {
+#pragma unroll 1
+                for (uint32_t a0 = 0; a0 < n_parts; a0 += 8) {
+                  float v[16];
+                  tmem_ld_8x2<part_cols(kN)>(from + a0 * part_cols(kN), v);
+                  if (n_parts - a0 < 8) {   // (parts that are not there)
+#pragma unroll
+                    for (uint32_t a = 1; a < 8; ++a)
+                      if (a0 + a >= n_parts) v[2 * a] = v[2 * a + 1] = 0.f;
+                  }
+                  float2 p[8];
+#pragma unroll
+                  for (uint32_t a = 0; a < 8; ++a) p[a] = make_float2(v[2 * a], v[2 * a + 1]);
+#pragma unroll
+                  for (uint32_t a = 0; a < 8; a += 4) {
+                    const float2 four = add2(add2(p[a], p[a + 1]), add2(p[a + 2], p[a + 3]));
+                    const float2 t = add2(s, four), d = sub2(t, s);
+                    lost = add2(lost, add2(sub2(s, sub2(t, d)), sub2(four, d)));
+                    s = t;
+                  }
+                }
+              });
+              // (an infinite sum has no remainder)
+              sum[0][0] = fabsf(s.x) <= 3.402823466e38f ? s.x + lost.x : s.x;
+              sum[0][1] = fabsf(s.y) <= 3.402823466e38f ? s.y + lost.y : s.y;
+              return;
+            }
+          }
+          each_slot([&](uint32_t from, uint32_t n_parts) {
+#pragma unroll 1
+            for (uint32_t a = 0; a < n_parts; ++a, from += part_cols(kN)) {
+              if constexpr (CH == 4) {
+                float v[4];
+                tmem_ld_4(from, v);
+                add(sum[0], v, 4);
+              } else if constexpr (CH == 8 && kGroups == 1) {
+                float v[8];
+                tmem_ld_8(from, v);
+                add(sum[0], v, 8);
+              } else if constexpr (CH == 16) {
+                float v[16];
+                tmem_ld_2x8(from, from + 8, v);
+                add(sum[0], v, 16);
+              } else {
+                static_assert(kN != 64 || (kGroups == 2 && CH == 8), "two groups of 8");
+                float v[16];
+                tmem_ld_2x8(from, from + HG * CH, v);
+                add(sum[0], v, 8);
+                add(sum[kGroups - 1], v + 8, 8);
+              }
+            }
+          });
+        }
+      };
       uint32_t image_no = 0;
       if (two) {
         if (w.u0 < w.u1) {
-          const uint32_t buf = acc % kBufs, from = lane_base + buf * kAcc;
-          const uint32_t half = nb / 2 / rounds_of(kN);                       // columns of a round that one threadblock finishes
+          constexpr uint32_t kRounds = rounds_of(kN);
+          const uint32_t half = nb / 2 / kRounds;                             // columns of a round that one threadblock finishes
           const uint32_t lanes = m64 ? 64u : kRowTile;                        // that hold sums
           float* own = kBig ? reinterpret_cast<float*>(x_ring) : sums;
           float* in = own + half * kRowTile;
           place(w.u0);
           if (epi == BOOST_EPI_ROPE_APPEND) row_table();
-          load_aux(rank * half, half, 0);
-          if (et == 0) {
-            if constexpr (!kBig) mbar_arrive_expect_tx(&xch_full, lanes * half * 4u);
-            wait(smem_u32(&acc_full[buf]), (acc / kBufs) & 1u);
-          }
-          named_barrier_sync(1, kEpiThreads);
-          tc_fence_after_sync();
-          for (uint32_t r = 0; r < rounds_of(kN); ++r, ++n_xch) {
-            const uint32_t mb = (2 * r + rank) * half, peer_mb = (2 * r + (rank ^ 1u)) * half;
-            if constexpr (kBig) {
-              // the peer may store here once this threadblock's products have read the activation slots
-              if (r) load_aux(mb, half, 0);
-              if (et == 0) {
-                mbar_arrive_expect_tx(&xch_full, lanes * half * 4u);
-                arrive_remote(mapa(smem_u32(&xch_free), rank ^ 1u));
-                wait(smem_u32(&xch_free), n_xch & 1u);
-              }
-              named_barrier_sync(1, kEpiThreads);
-            }
-            if (!__any_sync(0xFFFFFFFFu, s_abort != 0)) {   // the peer's columns
-              const uint32_t to = mapa(smem_u32(in), rank ^ 1u), bar = mapa(smem_u32(&xch_full), rank ^ 1u);
-              for (uint32_t c = hh * CH; c < half; c += HG * CH) {
-                float v[CH];
-                tmem_ld_cols<CH>(from + peer_mb + c, v);
+          // (from 128 rows on these operands wait in the chunk buffer, idle here, so that all rounds' are asked
+          // for ahead of the sums: about 1 % of a step)
+          float* const kept = sums + et;
 #pragma unroll
-                for (uint32_t j = 0; j < CH; ++j)
-                  if (holds) st_async_f32(to + ((c + j) * kRowTile + row) * 4u, v[j], bar);
+          for (uint32_t r = 0; r < (kParkSums ? kRounds : 1); ++r) {
+            load_aux((2 * r + rank) * half, half, 0);
+            if constexpr (kParkSums)
+#pragma unroll
+              for (uint32_t g = 0; g < G; ++g) {
+                kept[((r * G + g) * 2) * kEpiThreads] = aux_a[g];
+                kept[((r * G + g) * 2 + 1) * kEpiThreads] = aux_b[g];
+              }
+          }
+          if constexpr (!kBig)
+            if (et == 0) mbar_arrive_expect_tx(&xch_full, lanes * half * 4u);
+          accumulate();
+          if constexpr (kBig) {
+            // the peer may store here once this threadblock's products have read the activation slots
+            if (et == 0) {
+              mbar_arrive_expect_tx(&xch_full, lanes * half * kRounds * 4u);
+              arrive_remote(mapa(smem_u32(&xch_free), rank ^ 1u));
+              wait(smem_u32(&xch_free), n_xch & 1u);
+            }
+            named_barrier_sync(1, kEpiThreads);
+          }
+          if (!__any_sync(0xFFFFFFFFu, s_abort != 0)) {   // the peer's columns, of all rounds
+            const uint32_t to = mapa(smem_u32(in), rank ^ 1u), bar = mapa(smem_u32(&xch_full), rank ^ 1u);
+#pragma unroll
+            for (uint32_t i = 0; i < kGroups; ++i) {
+              const uint32_t share = column(i) / half, c = column(i) - share * half + (share >> 1) * half;
+              if ((share & 1u) == rank || share >= 2 * kRounds) continue;
+              float v[CH];
+              group_sums(i, v);
+              if (holds) {
+#pragma unroll
+                for (uint32_t e = 0; e < CH; ++e) st_async_f32(to + ((c + e) * kRowTile + row) * 4u, v[e], bar);
               }
             }
-            drain(from, mb, half, own);
-            if (r + 1 == rounds_of(kN)) release_acc(buf);
-            if (et == 0) wait(smem_u32(&xch_full), n_xch & 1u);
+          }
+          for (uint32_t r = 0; r < kRounds; ++r) {
+            const uint32_t mb = (2 * r + rank) * half;
+            if constexpr (kParkSums) {
+#pragma unroll
+              for (uint32_t g = 0; g < G; ++g) {
+                aux_a[g] = kept[((r * G + g) * 2) * kEpiThreads];
+                aux_b[g] = kept[((r * G + g) * 2 + 1) * kEpiThreads];
+              }
+            }
+#pragma unroll
+            for (uint32_t i = 0; i < kGroups; ++i) {   // this threadblock's columns of the round
+              const uint32_t share = column(i) / half, c = column(i) - share * half;
+              if (share != 2 * r + rank) continue;
+              float v[CH];
+              group_sums(i, v);
+              if (holds) {
+#pragma unroll
+                for (uint32_t e = 0; e < CH; ++e) own[(c + e) * kRowTile + row] = v[e];
+              }
+            }
+            if (kParkSums && r + 1 == kRounds) release_slot(parked);
+            if (et == 0 && r == 0) wait(smem_u32(&xch_full), n_xch & 1u);
             named_barrier_sync(1, kEpiThreads);
-            finish(own, in, mb, half, 0);
+            finish(own, in + r * half * kRowTile, mb, half, 0);
             if constexpr (kBig) {
               fence_proxy_async_smem();   // (the activation slots are written by TMA copies again)
               named_barrier_sync(1, kEpiThreads);
             }
           }
-          ++acc;
+          ++n_xch;
           image_no = 1;
         }
       } else {
+        constexpr uint32_t J = CW / (HG * CH);   // groups of a chunk
         const uint32_t n_chunks = (M_b + CW - 1) / CW;
-        for (uint32_t pa = w.u0; pa < w.u1; pa += w.run * kIpp, ++acc) {
-          const uint32_t buf = acc % kBufs, from = lane_base + buf * kAcc;
-          const uint32_t images = min(kIpp, (w.u1 - pa + w.run - 1) / w.run), n_steps = images * n_chunks;
-          place(pa);
+        for (uint32_t ua0 = w.u0; ua0 < w.u1; ua0 += w.run, ++image_no) {
+          place(ua0);
           if (epi == BOOST_EPI_ROPE_APPEND) row_table();
           load_aux(0, CW, 0);
-          if (et == 0) wait(smem_u32(&acc_full[buf]), (acc / kBufs) & 1u);
-          named_barrier_sync(1, kEpiThreads);
-          tc_fence_after_sync();
-          uint32_t img = 0, ch = 0;
-          for (uint32_t t = 0; t < n_steps; ++t) {
-            if (t) {
-              if (ch == 0) {
-                place(pa + img * w.run);
-                if (epi == BOOST_EPI_ROPE_APPEND) row_table();
+          accumulate();
+          for (uint32_t ch = 0; ch < n_chunks; ++ch) {
+            if (ch) load_aux(ch * CW, CW, 0);
+#pragma unroll
+            for (uint32_t j = 0; j < J; ++j) {
+              float v[CH];
+              group_sums(kParkSums ? ch * J + j : j, v);   // (not parked: there is one chunk)
+              if (holds) {
+#pragma unroll
+                for (uint32_t e = 0; e < CH; ++e) sums[(column(j) + e) * kRowTile + row] = v[e];
               }
-              load_aux(ch * CW, CW, 0);
             }
-            drain(from + img * kN, ch * CW, CW, sums);
-            if (t + 1 == n_steps) release_acc(buf);
+            if (kParkSums && ch + 1 == n_chunks) release_slot(parked);
             named_barrier_sync(1, kEpiThreads);
-            finish(sums, nullptr, ch * CW, CW, image_no + img);
+            finish(sums, nullptr, ch * CW, CW, image_no);
             named_barrier_sync(1, kEpiThreads);   // (the buffer and the row table are written again)
-            if (++ch == n_chunks) { ch = 0; ++img; }
           }
-          image_no += images;
         }
       }
       if (q.ssq_out) {   // images this worker does not have: their share of the statistics is zero
@@ -939,15 +1179,38 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
 uint32_t units_bound(uint32_t n_units, uint32_t W) { return (n_units + W - 1) / W; }
 uint32_t images_bound(uint32_t n_units, uint32_t W) { return (units_bound(n_units, W) + 15) / 16; }
 
+// k blocks of an accumulator.  Every hand-over costs the MMA warp 350 cycles and more (output product
+// at batch 32: 2800 of 14000 with eight), so parts are as long as the results allow:
+//   fp32 results   0.9 of the threadblocks' segments in the kernels of kernels_gemv.cu (two per SM up
+//                  to 128 rows, one above; none longer than a row tile's columns): the sums are then no
+//                  further from the exact ones than theirs.  Batches of 1 and 2, whose segments are
+//                  summed on CUDA cores there: a quarter of a block.
+//   bf16 results   at least 4096 columns (as many as those segments have at most): 4.4e-6 of the sum,
+//                  where the rounding behind it is 1.7e-3.
+// An even number (up to 16 rows a multiple of four: whole activation slots), or 1.
+uint32_t part_blocks_of(const PairPhase& q, uint32_t clusters, uint32_t M_b) {
+  const bool fp32 = q.epi == BOOST_EPI_PLAIN && q.y_dtype == 0;
+  if (fp32 && M_b <= 2) return 0;
+  const uint64_t blocks = (uint64_t)(q.n_units / kUnitsPerTile) * q.k_blocks, segments = (uint64_t)clusters * (M_b <= 128 ? 4 : 2);
+  uint32_t n = (uint32_t)(9 * (blocks < segments * q.k_blocks ? blocks : segments * q.k_blocks) / (10 * segments));
+  if (!fp32 && n < 64) n = 64;
+  const uint32_t unit = M_b <= 16 ? 4 : 2;
+  n = n / unit * unit;
+  if (n == 0) return 1;
+  const uint32_t own = (q.k_blocks + q.split - 1) / q.split, parts = (own + n - 1) / n;   // parts as even as they come
+  return ((own + parts - 1) / parts + unit - 1) / unit * unit;
+}
+
 // How a phase is cut.  Two threadblocks share the rows of a cluster, half of K each, where those rows
 // fit one image: little crosses between them, and the rows divide evenly (4096 rows over 74
 // clusters: 98.8 % of the SMs' time, over 148 threadblocks 86 %).  Longer products (gate / up, LM head)
 // have rows enough for every threadblock on its own (97 % and more) and nothing to exchange.
-void plan_phase(PairPhase& q, uint32_t clusters) {
+void plan_phase(PairPhase& q, uint32_t clusters, uint32_t M_b) {
   q.split = (q.k_blocks >= 2 && units_bound(q.n_units, clusters) <= 16) ? 2u : 1u;
   const uint32_t W = q.split == 2 ? clusters : 2 * clusters;
   q.image = units_bound(q.n_units, W) <= 8 ? 8u : 16u;
   q.max_images = images_bound(q.n_units, W);
+  q.part_blocks = part_blocks_of(q, clusters, M_b);
 }
 uint32_t ssq_parts_of(const PairPhase& q, uint32_t clusters) { return (q.split == 2 ? clusters : 2 * clusters) * q.max_images * (q.image / 8); }
 
@@ -970,10 +1233,10 @@ int launch_pair(PairParams& p, float* stats, size_t stats_bytes, int sms, cudaSt
   const int dev = boosth::device_slot();
   if (dev < 0) return BOOST_ERR_CUDA;
   PairState& st = states[dev];
-  // activation slots: more than a microsecond of a short product's stream (two k blocks per 310 ns); from
+  // activation slots: more than a microsecond of a short product's stream (a k block per 155 ns); from
   // 128 rows on about half of the shared memory, since the tiles are as large as the weight stages
   const uint32_t slot_bytes = x_blocks(kN) * p.nb * 128u;
-  const uint32_t x_budget = kN <= 16 ? 6 * slot_bytes : kN == 32 ? 4 * slot_bytes : kN == 64 ? 64u * 1024u : 96u * 1024u;
+  const uint32_t x_budget = kN <= 16 ? 3 * slot_bytes : kN == 32 ? 4 * slot_bytes : kN == 64 ? 64u * 1024u : 96u * 1024u;
   p.x_slots = x_budget / slot_bytes < kMaxXSlots ? x_budget / slot_bytes : kMaxXSlots;
   const uint32_t fixed = 2048u + p.x_slots * slot_bytes + sums_bytes(kN);
   p.n_stages = (smem_total(kN) - fixed) / kStageBytes;
@@ -1005,7 +1268,7 @@ int launch_pair(PairParams& p, float* stats, size_t stats_bytes, int sms, cudaSt
   uint32_t n_stats = 0;
   for (uint32_t i = 0; i < p.n_phases; ++i) {
     PairPhase& q = p.ph[i];
-    plan_phase(q, st.clusters);
+    plan_phase(q, st.clusters, p.M_b);
     for (int j = (int)i - 1; j >= 0; --j)
       if (q.ssq_in && key[j] == q.ssq_in) {
         q.ssq_in = p.ph[j].ssq_out;
@@ -1040,7 +1303,7 @@ uint32_t boosth::pair_split(uint32_t N, uint32_t K) {
   q.k_blocks = (K + 63) / 64;
   q.n_units = (N + kRowTile - 1) / kRowTile * kUnitsPerTile;
   const int sms = boosth::sm_count();
-  plan_phase(q, sms > 1 ? (uint32_t)sms / 2 : 1u);
+  plan_phase(q, sms > 1 ? (uint32_t)sms / 2 : 1u, 1);
   return q.split;
 }
 
