@@ -379,6 +379,9 @@ int boost_pack_weights_ex(const void* w_row_major /*device*/, uint32_t N, uint32
  *   y          device, row-major [M_b, N]; y_dtype 0 = fp32, 1 = bf16;
  *   residual   device bf16 [M_b, N] added before the final rounding, or NULL;
  *   workspace  device, >= boost_gemv_workspace_bytes(N, K, M_b).
+ * Everything is read after the kernels ahead of the call on the stream have finished: pages and page
+ * tables may have been written there.  (So has everything ahead of a decode step when its first
+ * product starts; after that a step reads weights while its own kernels run, none of which writes them.)
  * Products with rows of 1024 to 4096 columns (8192 where few rows leave two threadblocks to share
  * each) run on tcgen05 cut along the rows of the weight, in one launch without partial sums in memory.
  * Of the others, M_b <= 2 runs on CUDA cores with warp-shuffle reductions; larger batches use the

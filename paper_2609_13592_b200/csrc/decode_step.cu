@@ -186,7 +186,7 @@ int run_step(Launcher& L, const boost_llama_model_t* m, const boost_llama_scratc
   // host pages.
   const bool pair = !(boosth::two_queue_schedule() && has_host_weights(m));
   auto chain = [&](const boost_gemv_call_t* calls, uint32_t n) {
-    if (pair) return boosth::gemv_pair_launch(calls, n, B, s->gemv_ws, usable, tiles, slots.take(s, usable, n + 1), stream);
+    if (pair) return boosth::gemv_pair_launch(calls, n, B, s->gemv_ws, usable, tiles, slots.take(s, usable, n + 1), true, stream);
     uint32_t extra = 0;
     const int rc = boosth::gemv_chain_launch(calls, n, B, s->gemv_ws, usable, slots.take(s, usable, n + 1), true, tiles,
                                              stream, &extra);

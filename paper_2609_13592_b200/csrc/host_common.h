@@ -95,12 +95,12 @@ size_t gemv_partial_bytes(uint32_t N, uint32_t K, uint32_t M_b);
 int encode_activation_map(void* map, const void* x, uint32_t M_b, uint32_t K, uint32_t box_rows);
 
 // A chain of products whose split-K halves meet inside clusters (kernels_pair.cu); arguments as
-// gemv_chain_launch with early = true, weights with host pages are read in place.  The row
+// gemv_chain_launch, weights with host pages are read in place.  The row
 // statistics that pass from call to call live behind the workspace's counter area, in
 // pair_stats_bytes (an ssq_out pointer only names them; nothing is written there).
 size_t pair_stats_bytes(uint32_t N, uint32_t M_b);
 int gemv_pair_launch(const boost_gemv_call_t* calls, uint32_t n_calls, uint32_t M_b, void* workspace, size_t workspace_bytes,
-                     uint32_t header_row_tiles, uint32_t* sync_words, void* stream);
+                     uint32_t header_row_tiles, uint32_t* sync_words, bool early, void* stream);
 // How many threadblocks of a cluster share the columns of a product there (1 or 2).
 uint32_t pair_split(uint32_t N, uint32_t K);
 // The argument checks every weight product goes through.

@@ -1997,7 +1997,7 @@ extern "C" int boost_gemv_tiered(const void* const* w_page_ptr, const uint32_t* 
     boost_gemv_call_t c = {};
     c.w.page_ptr = w_page_ptr; c.w.order = w_order; c.w.n_pages = n_pages; c.w.n_host_pages = n_host_pages; c.w.N = N; c.w.K = K;
     c.x = x; c.y = y; c.y_dtype = y_dtype; c.residual = residual;
-    return boosth::gemv_pair_launch(&c, 1, M_b, workspace, workspace_bytes, 0, static_cast<uint32_t*>(workspace) + kWsBar, stream);
+    return boosth::gemv_pair_launch(&c, 1, M_b, workspace, workspace_bytes, 0, static_cast<uint32_t*>(workspace) + kWsBar, false, stream);
   }
   return boosth::gemv_tiered_launch(w_page_ptr, w_order, n_pages, n_host_pages, N, K, x, M_b, y, y_dtype,
                                     residual, workspace, workspace_bytes, nullptr, nullptr, 0, stream);

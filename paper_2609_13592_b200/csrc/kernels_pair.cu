@@ -83,6 +83,7 @@ struct PairPhase {
 
 struct PairParams {
   uint32_t n_phases, M_b, nb, n_stages, x_slots;   // nb: activation rows of a tile (the batch rounded up)
+  uint32_t early;  // weights and their page tables may be read while the kernel ahead on the stream still runs
   uint32_t* ws;    // workspace header
   uint32_t* bar;   // [0] threadblocks past their last wait, [1] phases finished, summed over the threadblocks; zero at rest
   PairPhase ph[kMaxPhases];
@@ -372,6 +373,10 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
   if (warp == 0 || warp == 3) {
     // ------------------------------------------------------------------ weight producers
     const uint32_t ring_a = smem_u32(ring), full_a = smem_u32(w_full), empty_a = smem_u32(w_empty);
+    if (!p.early) {
+      pdl_wait();
+      fence_proxy_async_all();   // pages written with ordinary stores are read through the TMA unit
+    }
     unsigned long long* const log = sched_log_of(p.ws);
     uint32_t stage = 0, parity = 1;
     bool my_turn = warp == 0;
@@ -727,9 +732,9 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
     // few sequences each.
     const uint32_t et = tid - kEpiWarp0 * 32, quarter = warp & 3u, hh = (warp - kEpiWarp0) >> 2;
     const uint32_t l128 = quarter * 32u + lane;   // tensor-memory lane
-    const uint32_t skip = et == 0 ? skip_arrivals_of(p.ws) : 0u;
     uint32_t as = 0, apar = 0, n_xch = 0;
     pdl_wait();
+    const uint32_t skip = et == 0 ? skip_arrivals_of(p.ws) : 0u;
     for (uint32_t ph = 0; ph < p.n_phases; ++ph) {
       const PairPhase& q = p.ph[ph];
       const Part w = part_of(q);
@@ -1308,7 +1313,7 @@ uint32_t boosth::pair_split(uint32_t N, uint32_t K) {
 }
 
 int boosth::gemv_pair_launch(const boost_gemv_call_t* calls, uint32_t n_calls, uint32_t M_b, void* workspace, size_t workspace_bytes,
-                             uint32_t header_row_tiles, uint32_t* sync_words, void* stream) {
+                             uint32_t header_row_tiles, uint32_t* sync_words, bool early, void* stream) {
   if (!calls || n_calls == 0 || n_calls > kMaxPhases || M_b == 0 || M_b > 256) return BOOST_ERR_INVALID;
   const int sms = boosth::sm_count();
   if (sms <= 0) return BOOST_ERR_CUDA;
@@ -1323,6 +1328,7 @@ int boosth::gemv_pair_launch(const boost_gemv_call_t* calls, uint32_t n_calls, u
   p.nb = n_class <= 32 ? n_class : M_b <= 128 ? (M_b + 15) / 16 * 16 : (M_b + 31) / 32 * 32;
   p.ws = static_cast<uint32_t*>(workspace);
   p.bar = sync_words;
+  p.early = early ? 1u : 0u;
   for (uint32_t i = 0; i < n_calls; ++i) {
     const boost_gemv_call_t& c = calls[i];
     const boost_gemv_epilogue_t& e = c.epilogue;
