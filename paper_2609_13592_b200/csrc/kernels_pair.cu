@@ -362,13 +362,10 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
     r.kb1 = two ? q.k_blocks * (rank + 1) / 2 : q.k_blocks;
     return r;
   };
-  // After a timeout the copies in flight must have landed before the shared memory goes away: a
-  // grace period far longer than a copy takes (their barriers may never complete).
-  auto grace = [&]() {
-    if (!s_abort) return;
-    const long long c0 = clock64();
-    while (clock64() - c0 < 100000) __nanosleep(1000);   // ~50 us
-  };
+  // Where a producer warp stands: the stage (activation slot) it would fill next, the parity of its wait for
+  // it, and whether it is this warp's turn.  Known at the end of the kernel too, for the wind-down.
+  uint32_t stage = 0, parity = 1;
+  bool my_turn = warp != 3;
 
   if (warp == 0 || warp == 3) {
     // ------------------------------------------------------------------ weight producers
@@ -378,8 +375,6 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
       fence_proxy_async_all();   // pages written with ordinary stores are read through the TMA unit
     }
     unsigned long long* const log = sched_log_of(p.ws);
-    uint32_t stage = 0, parity = 1;
-    bool my_turn = warp == 0;
     // Per stage: wait, announce the bytes, copy.  Everything else is kept out of the loop: the lanes
     // hold the pieces' addresses (part of the run x lower / upper rows; x k block of an image of 8), and
     // step through K on their own.
@@ -445,7 +440,6 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
     };
     for (uint32_t ph = 0; ph < p.n_phases; ++ph)
       if (!produce(p.ph[ph], ph)) break;
-    grace();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ activation producer
     // Up to 32 rows: 16-byte copies through the load/store path (the TMA unit works in order, and an
@@ -458,7 +452,7 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
       __syncwarp();
     }
     pdl_wait();
-    uint32_t xs = 0, parity = 1;
+    uint32_t& xs = stage;
     auto produce = [&](const PairPhase& q, uint32_t ph) -> bool {
       const Part w = part_of(q);
       const uint32_t K = q.K, run = w.run;
@@ -531,7 +525,6 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
       if (!produce(p.ph[ph], ph)) break;
     }
     if constexpr (!kTmaX) cp_async_wait_all();   // (nothing in flight when the shared memory goes away)
-    else grace();
   } else if (warp == 2) {
     // ------------------------------------------------------------------ MMA issue
     // This warp's instruction latency is what bounds a product whose operands are in place (measured with
@@ -718,12 +711,6 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
     };
     for (uint32_t ph = 0; ph < p.n_phases; ++ph)
       if (!multiply_phase(p.ph[ph])) break;
-    if (s_abort) {
-      // nothing may be in the tensor cores' pipeline when its operands and accumulators go away
-      if (elect_one()) commit(smem_u32(&drained));
-      __syncwarp();
-      mbar_wait(&drained, 0, status);
-    }
   } else if (warp >= kEpiWarp0) {
     // ------------------------------------------------------------------ epilogue
     // An image's accumulators are added up as they come, and the sums go to shared memory (half of the
@@ -743,7 +730,9 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
       const uint32_t epi = q.epi, N = q.N, M_b = p.M_b;
       if (ph > 0) {   // (one thread polls, the others wait in the hardware barrier)
         if (et == 0) wait(smem_u32(&go), (ph - 1) & 1u);
-        named_barrier_sync(1, kEpiThreads);
+        // After a wait that gave up, everybody leaves before the next phase: a barrier whose peer never
+        // came is not armed a second time.
+        if (named_barrier_or(1, kEpiThreads, s_abort != 0)) break;
       }
       if (q.ssq_in && w.u0 < w.u1) {
         // row scales of this phase's activations: the parts in kGroups interleaved groups, then the groups in order
@@ -1175,10 +1164,30 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
+  if (s_abort) {
+    // A wait gave up somewhere (every role is past its last wait now, so nobody starts anything new): nothing
+    // may be in the tensor cores' pipeline or on its way to shared memory when that goes away.  Each
+    // issuer waits, as long as any other wait, for what it has started.  (A fixed time would not do: over
+    // the host link the copies in flight of all threadblocks are a third of a millisecond.)
+    if (warp == 2) {
+      if (elect_one()) commit(smem_u32(&drained));
+      __syncwarp();
+      mbar_wait(&drained, 0, status);
+    } else if (warp < kEpiWarp0 && (warp != 1 || kTmaX)) {
+      // the last use of every stage, backwards from the next one (uses before the first count as landed)
+      const uint32_t n = warp == 1 ? x_slots : n_stages;
+      for (uint32_t i = 0; i < n; ++i) {
+        if (stage == 0) { stage = n; parity ^= 1u; }
+        --stage;
+        if (warp != 1) my_turn = !my_turn;
+        if (my_turn) mbar_wait(warp == 1 ? &x_full[stage] : &w_full[stage], parity ^ 1u, status);
+      }
+    }
+    __syncthreads();
+    // Nor may the peer store here any more.  (Without a failed wait, what it stores and signals here has been waited for.)
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
   if (warp == 2) tmem_dealloc(tmem, tmem_cols(kN));
-  // Nobody gives up its shared memory while the peer may still store into it.  What the peer stores and
-  // signals here has been waited for above, unless a wait gave up.
-  if (s_abort) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 uint32_t units_bound(uint32_t n_units, uint32_t W) { return (n_units + W - 1) / W; }

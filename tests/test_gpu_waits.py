@@ -119,3 +119,41 @@ def test_missing_partial_sum_times_out_in_tile_finish(dev):
     torch.cuda.synchronize()
     again = run()
     assert int(header[0]) == 0 and torch.equal(again, good)
+
+
+@pytest.mark.parametrize("n_seq,on_host", [(2, False), (12, True), (24, False), (60, True), (100, False), (140, True)])
+def test_missing_arrival_in_a_step_times_out_and_the_step_returns(dev, n_seq, on_host):
+    """The cluster kernel that runs a decode step (every batch class; weights in HBM, or all of them on
+    their way over the host link when the waits give up): threadblock 0 keeps its arrivals between
+    products to itself, the others' waits run out, every launch of the step comes back with the time-out on
+    record, and after a zero-fill the step gives the bits it gave before."""
+    from tests.test_gpu_decode import build_decoder, first_page_on_host, load_caches
+    cfg = dict(n_layers=2, hidden=512, ffn=1024, n_q_heads=4, n_kv_heads=2, head_dim=128, vocab=3000)
+    w = synth.llama_weights(cfg, seed=9, std=0.03)
+    n_pool_blocks = 1024
+    dec = build_decoder(dev, cfg, w, n_pool_blocks, 0, 0.0, n_seq, 4, weight_tier=first_page_on_host if on_host else None)
+    rng = np.random.default_rng(n_seq)
+    ctx = rng.integers(1, 64, size=n_seq).astype(np.int32)
+    table = rng.permutation(n_pool_blocks)[:n_seq * 4].reshape(n_seq, 4).astype(np.int32)
+    tokens = rng.integers(0, cfg["vocab"], size=n_seq).astype(np.int32)
+    cache = [synth.normal_bf16((2, n_pool_blocks, 16, 128), 1.0, 50 + li) for li in range(2)]
+    load_caches(dev, dec, cache, cache)
+    ws_t = dec._gemv_ws_t
+    header = ws_t[dec._gemv_ws_ptr - ws_t.data_ptr():][:64].view(torch.int32)
+
+    def run():
+        dec.step_host(tokens, table, ctx, np.zeros(n_seq, np.int32))     # waits for the stream: nothing hangs
+        return [dec.buf[name][:n_seq].clone() for name in ("logits", "h")]
+
+    good = run()
+    assert int(header[0]) == 0 and bool(torch.isfinite(good[0]).all()) and float(good[0].abs().sum()) > 0
+    header[WS_WAIT_LIMIT_WORD] = 2_000_000
+    header[WS_SKIP_ARRIVALS_WORD] = 1
+    torch.cuda.synchronize()
+    run()                                                                # outputs of this step mean nothing
+    assert int(header[0]) & 1 == 1
+    ws_t.zero_()
+    torch.cuda.synchronize()
+    again = run()
+    assert dec.status_words() == [0, 0]
+    assert all(torch.equal(a, b) for a, b in zip(again, good))
