@@ -448,8 +448,8 @@ typedef struct {
 
 /* Chooses between the two tensor-core kernels of the products that meet in L2 (fused and chained
  * products, rows of more than 8192 or fewer than 1024 columns, the two-queue schedule); at any other
- * value than the default a plain boost_gemv_tiered takes one of those kernels as well, at the
- * default mostly the cluster kernel (its threadblocks pair up in clusters that add up halves of
+ * value than the default a plain boost_gemv_tiered and a decode step take one of those kernels as well, at the
+ * default the cluster kernel (its threadblocks pair up in clusters that add up halves of
  * the columns in distributed shared memory).  Batches of at least m_b rows run on the tcgen05 kernel (operands from shared memory through
  * matrix descriptors, accumulators in tensor memory), smaller ones down to 3 rows on the
  * mma.sync kernel; 1 and 2 rows always use the CUDA cores.  Process-wide; the results of the

@@ -181,10 +181,10 @@ int run_step(Launcher& L, const boost_llama_model_t* m, const boost_llama_scratc
     if (!L.ok()) return L.rc;
   }
   // The kernel whose split-K halves meet inside clusters (8B-shaped step against the kernels of
-  // kernels_gemv.cu: batch 1 3564 -> 3177 us, 32 5366 -> 4736; 16 layers at batch 128 4368 -> 4162; 8
-  // layers at batch 250 2925 -> 2705), except under the two-queue schedule, which is about weights with
-  // host pages.
-  const bool pair = !(boosth::two_queue_schedule() && has_host_weights(m));
+  // kernels_gemv.cu: 6 layers at batch 1 808 -> 686 us, 8 845 -> 709, 32 963 -> 802, 128 1458 -> 1330, 250 2318 ->
+  // 2045), except where a process-wide switch asks for one of those kernels (the two-queue schedule: for
+  // weights with host pages).
+  const bool pair = boosth::cluster_products(has_host_weights(m));
   auto chain = [&](const boost_gemv_call_t* calls, uint32_t n) {
     if (pair) return boosth::gemv_pair_launch(calls, n, B, s->gemv_ws, usable, tiles, slots.take(s, usable, n + 1), true, stream);
     uint32_t extra = 0;

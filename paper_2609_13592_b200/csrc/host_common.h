@@ -105,8 +105,8 @@ int gemv_pair_launch(const boost_gemv_call_t* calls, uint32_t n_calls, uint32_t 
 uint32_t pair_split(uint32_t N, uint32_t K);
 // The argument checks every weight product goes through.
 int gemv_check_call(const boost_gemv_call_t& call, uint32_t M_b, void* workspace, size_t workspace_bytes, uint32_t header_row_tiles);
-// Whether boost_gemv_set_tier_schedule asks for the two-queue schedule (weights with host pages).
-bool two_queue_schedule();
+// Whether the process-wide switches leave products (with host pages or without) to the cluster kernel.
+bool cluster_products(bool host_pages);
 
 // Launch check: picks up configuration errors of the launch just made.
 inline int check_launch() { return check(cudaGetLastError()); }

@@ -1715,8 +1715,6 @@ int launch_gemv_tc(const ChainParams& chain, int sms, cudaStream_t stream, uint3
 
 }  // namespace
 
-bool boosth::two_queue_schedule() { return g_tier_schedule != 0; }
-
 // The driver's encoder is looked up at run time (no link-time dependency on the driver library).
 int boosth::encode_activation_map(void* map, const void* x, uint32_t M_b, uint32_t K, uint32_t box_rows) {
   using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -1983,8 +1981,12 @@ int boosth::gemv_chain_launch(const boost_gemv_call_t* calls, uint32_t n_calls, 
 //   - one of the process-wide switches that choose among the kernels above is not at its default.
 constexpr uint32_t kPairMaxDepth = 4096, kPairMinColumns = 1024;
 
+bool boosth::cluster_products(bool host_pages) {
+  return g_tc_min_batch == kTcMinBatchDefault && g_end_combine && !(g_tier_schedule && host_pages);
+}
+
 static bool pair_takes(uint32_t N, uint32_t K, size_t n_host_pages) {
-  if (g_tc_min_batch != kTcMinBatchDefault || !g_end_combine || (g_tier_schedule && n_host_pages)) return false;
+  if (!boosth::cluster_products(n_host_pages != 0)) return false;
   return K >= kPairMinColumns && K <= kPairMaxDepth * boosth::pair_split(N, K);
 }
 

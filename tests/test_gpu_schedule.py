@@ -176,3 +176,41 @@ def test_gemv_chain_and_attention_schedule(dev, two_queues):
                       for blk in table[b, :(c + 15) // 16] for g in range(hkv))
     assert int(recs["host_bytes"].sum()) == host_chunks * 8192 and host_chunks > 0
     pool.close()
+
+
+@pytest.mark.parametrize("n_seq,switched", [(2, False), (20, False), (70, False), (200, False), (20, True)])
+def test_step_schedule(dev, n_seq, switched):
+    """The log of a decode step: one record per threadblock and product on the cluster kernel, with every
+    byte of every weight once and the host pages' bytes as such.  switched: a process-wide switch of the
+    split-K kernels reaches a step too (their records name the warp that streamed)."""
+    from tests.test_gpu_decode import build_decoder, load_caches
+    cfg = dict(n_layers=1, hidden=1024, ffn=2048, n_q_heads=4, n_kv_heads=2, head_dim=128, vocab=6000)
+    w = synth.llama_weights(cfg, seed=4, std=0.03)
+    every_third = lambda name, layer, n_pages: (np.arange(n_pages) % 3 == 0).astype(np.uint8)
+    dec = build_decoder(dev, cfg, w, 1024, 0, 0.0, n_seq, 4, weight_tier=every_third)
+    cache = [synth.normal_bf16((2, 1024, 16, 128), 1.0, 5)]
+    load_caches(dev, dec, cache, cache)
+    rng = np.random.default_rng(1)
+    args = (rng.integers(0, cfg["vocab"], size=n_seq).astype(np.int32),
+            rng.permutation(1024)[:n_seq * 4].reshape(n_seq, 4).astype(np.int32),
+            rng.integers(1, 64, size=n_seq).astype(np.int32), np.zeros(n_seq, np.int32))
+    try:
+        B.boost_gemv_set_end_combine(not switched)
+        dec.step_host(*args)
+        want = dec.buf["logits"][:n_seq].clone()
+        log = make_log(dev, 8192)
+        attach(dec._gemv_ws_t, dec._gemv_ws_ptr, log)
+        dec.step_host(*args)
+    finally:
+        B.boost_gemv_set_end_combine(True)
+    assert torch.equal(dec.buf["logits"][:n_seq], want)                    # logging changes no result
+    recs, _ = check_against_oracle(log, B.SCHED_KIND_GEMV, 64, 1000, 1 / 3)
+    ly = dec.layers[0]
+    for ph, mats in enumerate([(ly["wqkv"], ly["wo"]), (ly["wgu"],), (ly["wd"],), (dec.lm_head,)]):   # (the first product is a launch of its own)
+        mine = recs[(recs["kind_phase"] >> 8) == ph]
+        assert int(mine["bytes"].sum()) == sum(m.layout["n_row_tiles"] * m.layout["k_blocks"] * 16384 for m in mats)
+        pages = [(int(p), m.layout["n_row_tiles"] * m.layout["k_blocks"]) for m in mats for p in np.flatnonzero(m.buf.tier)]
+        assert int(mine["host_bytes"].sum()) == sum(min(128, blocks - 128 * p) * 16384 for p, blocks in pages) > 0
+        assert (mine["t_consumed"] > mine["t_request"]).all()
+        assert bool((mine["cta_warp"] >> 24).any()) == switched
+    assert dec.status_words() == [0, 0]
