@@ -446,11 +446,11 @@ typedef struct {
   const void* const* v_page_ptr2; /* device or NULL */
 } boost_gemv_epilogue_t;
 
-/* Chooses between the two tensor-core kernels of the products that meet in L2 (fused and chained
- * products, rows of more than 8192 or fewer than 1024 columns, the two-queue schedule); at any other
- * value than the default a plain boost_gemv_tiered and a decode step take one of those kernels as well, at the
- * default the cluster kernel (its threadblocks pair up in clusters that add up halves of
- * the columns in distributed shared memory).  Batches of at least m_b rows run on the tcgen05 kernel (operands from shared memory through
+/* Chooses between the two tensor-core kernels of the products that meet in L2 (products with row
+ * statistics, SwiGLU or RoPE epilogues, rows of more than 8192 or fewer than 1024 columns, the
+ * two-queue schedule); at any other value than the default plain products and decode steps take
+ * one of those kernels as well, at the default the cluster kernel (its threadblocks pair up in
+ * clusters that add up halves of the columns in distributed shared memory).  Batches of at least m_b rows run on the tcgen05 kernel (operands from shared memory through
  * matrix descriptors, accumulators in tensor memory), smaller ones down to 3 rows on the
  * mma.sync kernel; 1 and 2 rows always use the CUDA cores.  Process-wide; the results of the
  * two tensor-core kernels agree to fp32 rounding.  Default 33 (measured crossover on B200).  The paper has no counterpart
@@ -481,7 +481,7 @@ int boost_gemv_set_end_combine(uint32_t on);
  * rounding (other partial sums).  Process-wide; for measurement, tests and the comparison with the paper's schedule. */
 int boost_gemv_set_tier_schedule(uint32_t two_queues);
 
-/* boost_gemv_tiered with an epilogue descriptor (NULL = plain). */
+/* boost_gemv_tiered with an epilogue descriptor (NULL, or PLAIN without row statistics: the same call). */
 int boost_gemv_tiered_fused(const void* const* w_page_ptr /*device*/, const uint32_t* w_order /*device*/,
                             size_t n_pages, size_t n_host_pages, uint32_t N, uint32_t K,
                             const void* x /*device*/, uint32_t M_b, void* y /*device*/, int y_dtype,
@@ -510,7 +510,8 @@ typedef struct {
 
 /* A chain of 1..4 weight products in ONE launch, each of which may take what the previous
  * ones wrote (as its x, its residual or its row statistics): the results equal those of the
- * same calls of boost_gemv_tiered_fused made one after the other.  Sec. 2.1 describes decode as
+ * same calls of boost_gemv_tiered_fused made one after the other, bit for bit.  (A chain that mixes
+ * plain products of the cluster kernel with others is a launch for each run of either kind.)  Sec. 2.1 describes decode as
  * a chain of weight-streaming products; because weights do not depend on activations, the
  * persistent threadblocks stream the next product's weight pages (both tiers, host pages
  * first, as in boost_gemv_tiered) while the tail of the current product drains, and meet at

@@ -1817,15 +1817,6 @@ extern "C" size_t boost_gemv_workspace_bytes(uint32_t N, uint32_t K, uint32_t M_
   return boosth::gemv_header_bytes(lay.n_row_tiles) + boosth::gemv_partial_bytes(N, K, M_b);
 }
 
-extern "C" int boost_gemv_tiered_fused(const void* const* w_page_ptr, const uint32_t* w_order,
-                                       size_t n_pages, size_t n_host_pages, uint32_t N, uint32_t K,
-                                       const void* x, uint32_t M_b, void* y, int y_dtype,
-                                       const void* residual, const boost_gemv_epilogue_t* epilogue,
-                                       void* workspace, size_t workspace_bytes, void* stream) {
-  return boosth::gemv_tiered_launch(w_page_ptr, w_order, n_pages, n_host_pages, N, K, x, M_b, y, y_dtype,
-                                    residual, workspace, workspace_bytes, epilogue, nullptr, 0, stream);
-}
-
 namespace {
 
 // Checks one product's arguments and fills its kernel parameters.  `header` = bytes of the
@@ -1972,8 +1963,9 @@ int boosth::gemv_chain_launch(const boost_gemv_call_t* calls, uint32_t n_calls, 
   return launch_routed(c, M_b, stream, extra_launches);
 }
 
-// A plain product on its own goes to the cluster kernel (kernels_pair.cu): one launch instead of the
-// product and its combine, no partial sums in memory.  Not where
+// A plain product (no row statistics in or out) goes to the cluster kernel (kernels_pair.cu), whichever
+// entry it comes through: one launch instead of the product and its combine, no partial sums in
+// memory.  Not where
 //   - a threadblock's share of the columns would be more than kPairMaxDepth: longer rows on their own
 //     are not measured on it (in a step they are: the down product's 7168);
 //   - the rows are short: a threadblock's time is then its epilogue, and the kernels above finish
@@ -1985,9 +1977,26 @@ bool boosth::cluster_products(bool host_pages) {
   return g_tc_min_batch == kTcMinBatchDefault && g_end_combine && !(g_tier_schedule && host_pages);
 }
 
-static bool pair_takes(uint32_t N, uint32_t K, size_t n_host_pages) {
-  if (!boosth::cluster_products(n_host_pages != 0)) return false;
-  return K >= kPairMinColumns && K <= kPairMaxDepth * boosth::pair_split(N, K);
+static bool cluster_takes(const boost_gemv_call_t& c) {
+  if (c.has_epilogue && (c.epilogue.mode != BOOST_EPI_PLAIN || c.epilogue.ssq_in || c.epilogue.ssq_out)) return false;
+  if (c.w.N == 0 || c.w.K < kPairMinColumns || !boosth::cluster_products(c.w.n_host_pages != 0)) return false;
+  return c.w.K <= kPairMaxDepth * boosth::pair_split(c.w.N, c.w.K);
+}
+
+extern "C" int boost_gemv_tiered_fused(const void* const* w_page_ptr, const uint32_t* w_order,
+                                       size_t n_pages, size_t n_host_pages, uint32_t N, uint32_t K,
+                                       const void* x, uint32_t M_b, void* y, int y_dtype,
+                                       const void* residual, const boost_gemv_epilogue_t* epilogue,
+                                       void* workspace, size_t workspace_bytes, void* stream) {
+  boost_gemv_call_t c = {};
+  c.w.page_ptr = w_page_ptr; c.w.order = w_order; c.w.n_pages = n_pages; c.w.n_host_pages = n_host_pages; c.w.N = N; c.w.K = K;
+  c.x = x; c.y = y; c.y_dtype = y_dtype; c.residual = residual;
+  c.has_epilogue = epilogue != nullptr;
+  if (epilogue) c.epilogue = *epilogue;
+  if (workspace && cluster_takes(c))
+    return boosth::gemv_pair_launch(&c, 1, M_b, workspace, workspace_bytes, 0, static_cast<uint32_t*>(workspace) + kWsBar, false, stream);
+  return boosth::gemv_tiered_launch(w_page_ptr, w_order, n_pages, n_host_pages, N, K, x, M_b, y, y_dtype,
+                                    residual, workspace, workspace_bytes, epilogue, nullptr, 0, stream);
 }
 
 extern "C" int boost_gemv_tiered(const void* const* w_page_ptr, const uint32_t* w_order,
@@ -1995,14 +2004,8 @@ extern "C" int boost_gemv_tiered(const void* const* w_page_ptr, const uint32_t* 
                                  const void* x, uint32_t M_b, void* y, int y_dtype,
                                  const void* residual, void* workspace, size_t workspace_bytes,
                                  void* stream) {
-  if (workspace && pair_takes(N, K, n_host_pages)) {
-    boost_gemv_call_t c = {};
-    c.w.page_ptr = w_page_ptr; c.w.order = w_order; c.w.n_pages = n_pages; c.w.n_host_pages = n_host_pages; c.w.N = N; c.w.K = K;
-    c.x = x; c.y = y; c.y_dtype = y_dtype; c.residual = residual;
-    return boosth::gemv_pair_launch(&c, 1, M_b, workspace, workspace_bytes, 0, static_cast<uint32_t*>(workspace) + kWsBar, false, stream);
-  }
-  return boosth::gemv_tiered_launch(w_page_ptr, w_order, n_pages, n_host_pages, N, K, x, M_b, y, y_dtype,
-                                    residual, workspace, workspace_bytes, nullptr, nullptr, 0, stream);
+  return boost_gemv_tiered_fused(w_page_ptr, w_order, n_pages, n_host_pages, N, K, x, M_b, y, y_dtype, residual, nullptr, workspace,
+                                 workspace_bytes, stream);
 }
 
 extern "C" size_t boost_gemv_chain_workspace_bytes(const boost_gemv_call_t* calls, uint32_t n_calls, uint32_t M_b) {
@@ -2034,7 +2037,25 @@ extern "C" int boost_gemv_tiered_chain(const boost_gemv_call_t* calls, uint32_t 
   // call reuse the workspace on the same stream: that call's threadblocks may become resident
   // while this one drains, so none of them may touch the words before this launch has completed
   // (early = false: the weight warps also wait for the preceding kernel).
-  return boosth::gemv_chain_launch(calls, n_calls, M_b, workspace, usable, sync_words, false, 0, stream);
+  // Runs of plain products that the cluster kernel takes, and runs of the others, are a launch each: every
+  // product is computed as on its own.  All arguments are checked before the first launch.
+  uint32_t tiles = 0;
+  for (uint32_t i = 0; i < n_calls; ++i) {
+    const uint32_t t = (calls[i].w.N + kBlockRows - 1) / kBlockRows;
+    tiles = t > tiles ? t : tiles;
+  }
+  for (uint32_t i = 0; i < n_calls; ++i) {
+    const int rc = boosth::gemv_check_call(calls[i], M_b, workspace, usable, tiles);
+    if (rc != BOOST_OK) return rc;
+  }
+  for (uint32_t i = 0, n; i < n_calls; i += n) {
+    const bool cluster = cluster_takes(calls[i]);
+    for (n = 1; i + n < n_calls && cluster_takes(calls[i + n]) == cluster; ++n) {}
+    const int rc = cluster ? boosth::gemv_pair_launch(calls + i, n, M_b, workspace, usable, tiles, sync_words + 16 * i, false, stream)
+                           : boosth::gemv_chain_launch(calls + i, n, M_b, workspace, usable, sync_words + 16 * i, false, tiles, stream);
+    if (rc != BOOST_OK) return rc;
+  }
+  return BOOST_OK;
 }
 
 // Routing threshold between the two tensor-core kernels (measurement and tests).
