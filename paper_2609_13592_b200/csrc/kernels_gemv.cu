@@ -1970,6 +1970,7 @@ int boosth::gemv_chain_launch(const boost_gemv_call_t* calls, uint32_t n_calls, 
 //     are not measured on it (in a step they are: the down product's 7168);
 //   - the rows are short: a threadblock's time is then its epilogue, and the kernels above finish
 //     tiles from tensor memory;
+//   - y overlaps x: a threadblock writes its rows while others still read x;
 //   - one of the process-wide switches that choose among the kernels above is not at its default.
 constexpr uint32_t kPairMaxDepth = 4096, kPairMinColumns = 1024;
 
@@ -1977,10 +1978,13 @@ bool boosth::cluster_products(bool host_pages) {
   return g_tc_min_batch == kTcMinBatchDefault && g_end_combine && !(g_tier_schedule && host_pages);
 }
 
-static bool cluster_takes(const boost_gemv_call_t& c) {
+static bool cluster_takes(const boost_gemv_call_t& c, uint32_t M_b) {
   if (c.has_epilogue && (c.epilogue.mode != BOOST_EPI_PLAIN || c.epilogue.ssq_in || c.epilogue.ssq_out)) return false;
   if (c.w.N == 0 || c.w.K < kPairMinColumns || !boosth::cluster_products(c.w.n_host_pages != 0)) return false;
-  return c.w.K <= kPairMaxDepth * boosth::pair_split(c.w.N, c.w.K);
+  if (c.w.K > kPairMaxDepth * boosth::pair_split(c.w.N, c.w.K)) return false;
+  const uint8_t *x = static_cast<const uint8_t*>(c.x), *y = static_cast<const uint8_t*>(c.y);
+  const size_t x_bytes = (size_t)M_b * c.w.K * 2, y_bytes = (size_t)M_b * c.w.N * (c.y_dtype == 0 ? 4 : 2);
+  return x + x_bytes <= y || y + y_bytes <= x;
 }
 
 extern "C" int boost_gemv_tiered_fused(const void* const* w_page_ptr, const uint32_t* w_order,
@@ -1993,7 +1997,7 @@ extern "C" int boost_gemv_tiered_fused(const void* const* w_page_ptr, const uint
   c.x = x; c.y = y; c.y_dtype = y_dtype; c.residual = residual;
   c.has_epilogue = epilogue != nullptr;
   if (epilogue) c.epilogue = *epilogue;
-  if (workspace && cluster_takes(c))
+  if (workspace && cluster_takes(c, M_b))
     return boosth::gemv_pair_launch(&c, 1, M_b, workspace, workspace_bytes, 0, static_cast<uint32_t*>(workspace) + kWsBar, false, stream);
   return boosth::gemv_tiered_launch(w_page_ptr, w_order, n_pages, n_host_pages, N, K, x, M_b, y, y_dtype,
                                     residual, workspace, workspace_bytes, epilogue, nullptr, 0, stream);
@@ -2049,8 +2053,8 @@ extern "C" int boost_gemv_tiered_chain(const boost_gemv_call_t* calls, uint32_t 
     if (rc != BOOST_OK) return rc;
   }
   for (uint32_t i = 0, n; i < n_calls; i += n) {
-    const bool cluster = cluster_takes(calls[i]);
-    for (n = 1; i + n < n_calls && cluster_takes(calls[i + n]) == cluster; ++n) {}
+    const bool cluster = cluster_takes(calls[i], M_b);
+    for (n = 1; i + n < n_calls && cluster_takes(calls[i + n], M_b) == cluster; ++n) {}
     const int rc = cluster ? boosth::gemv_pair_launch(calls + i, n, M_b, workspace, usable, tiles, sync_words + 16 * i, false, stream)
                            : boosth::gemv_chain_launch(calls + i, n, M_b, workspace, usable, sync_words + 16 * i, false, tiles, stream);
     if (rc != BOOST_OK) return rc;
