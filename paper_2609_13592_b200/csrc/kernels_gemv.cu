@@ -1981,7 +1981,7 @@ bool boosth::cluster_products(bool host_pages) {
 static bool cluster_takes(const boost_gemv_call_t& c, uint32_t M_b) {
   if (c.has_epilogue && (c.epilogue.mode != BOOST_EPI_PLAIN || c.epilogue.ssq_in || c.epilogue.ssq_out)) return false;
   if (c.w.N == 0 || c.w.K < kPairMinColumns || !boosth::cluster_products(c.w.n_host_pages != 0)) return false;
-  if (c.w.K > kPairMaxDepth * boosth::pair_split(c.w.N, c.w.K)) return false;
+  if (c.w.K > kPairMaxDepth * boosth::pair_split(c.w.N, c.w.K, M_b)) return false;
   const uint8_t *x = static_cast<const uint8_t*>(c.x), *y = static_cast<const uint8_t*>(c.y);
   const size_t x_bytes = (size_t)M_b * c.w.K * 2, y_bytes = (size_t)M_b * c.w.N * (c.y_dtype == 0 ? 4 : 2);
   return x + x_bytes <= y || y + y_bytes <= x;

@@ -40,6 +40,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "device_common.cuh"
 #include "host_common.h"
 
@@ -1228,25 +1230,69 @@ void plan_phase(PairPhase& q, uint32_t clusters, uint32_t M_b) {
 }
 uint32_t ssq_parts_of(const PairPhase& q, uint32_t clusters) { return (q.split == 2 ? clusters : 2 * clusters) * q.max_images * (q.image / 8); }
 
-struct PairState {
-  bool configured = false;
-  uint32_t clusters = 0;   // clusters of two the device holds at once
-};
-
 // Shared memory of an instantiation.  More than half an SM, so that no two threadblocks of this kernel
 // share one (the grid counts on one threadblock per SM).  Up to 32 rows a threadblock of the
 // attention kernel fits beside it (measured, 3-layer step at batch 1 / 32: 493 / 683 us with 145 KiB,
 // 507 / 685 with 180); above, the activation tiles need the room.
 constexpr uint32_t smem_total(uint32_t n) { return (n <= 32 ? 147u : 214u) * 1024u; }
 
+// Clusters of two that the current device holds at once, one threadblock per SM (0: none, or an error, which
+// is left in `rc`).  Set up once per device; every rule about how a product is cut starts from here.
+template <uint32_t kN>
+uint32_t clusters_of(int& rc) {
+  static std::atomic<uint32_t> known[boosth::kMaxDevices];   // count + 1; threads that meet here find the same
+  const int dev = boosth::device_slot(), sms = boosth::sm_count();
+  rc = dev < 0 || sms <= 0 ? BOOST_ERR_CUDA : BOOST_OK;
+  if (rc != BOOST_OK) return 0;
+  const uint32_t seen = known[dev].load(std::memory_order_acquire);
+  if (seen) return seen - 1;
+  rc = boosth::check(cudaFuncSetAttribute(gemv_pair_kernel<kN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_total(kN)));
+  if (rc != BOOST_OK) return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2);
+  cfg.blockDim = dim3(threads_of(kN));
+  cfg.dynamicSmemBytes = smem_total(kN);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  rc = boosth::check(cudaOccupancyMaxActiveClusters(&n, gemv_pair_kernel<kN>, &cfg));
+  if (rc != BOOST_OK) return 0;
+  const uint32_t clusters = (uint32_t)n < (uint32_t)sms / 2 ? (uint32_t)n : (uint32_t)sms / 2;
+  known[dev].store(clusters + 1, std::memory_order_release);
+  return clusters;
+}
+
+uint32_t batch_class(uint32_t M_b) { return M_b <= 8 ? 8 : M_b <= 16 ? 16 : M_b <= 32 ? 32 : M_b <= 64 ? 64 : M_b <= 128 ? 128 : 256; }
+
+// The same by batch, for sizes and rules (without a device: a B200's 74).
+uint32_t clusters_for(uint32_t M_b) {
+  int rc = BOOST_OK;
+  uint32_t n = 0;
+  switch (boosth::device_slot() < 0 ? 0 : batch_class(M_b)) {
+    case 0: break;
+    case 8: n = clusters_of<8>(rc); break;
+    case 16: n = clusters_of<16>(rc); break;
+    case 32: n = clusters_of<32>(rc); break;
+    case 64: n = clusters_of<64>(rc); break;
+    case 128: n = clusters_of<128>(rc); break;
+    default: n = clusters_of<256>(rc);
+  }
+  return n ? n : 74;
+}
+
 // Row statistics between the phases of one launch live in two buffers of the workspace; a phase's
 // ssq_in is matched to the earlier phase that produces it by the caller's ssq_out pointer.
 template <uint32_t kN>
-int launch_pair(PairParams& p, float* stats, size_t stats_bytes, int sms, cudaStream_t stream) {
-  static PairState states[boosth::kMaxDevices];
-  const int dev = boosth::device_slot();
-  if (dev < 0) return BOOST_ERR_CUDA;
-  PairState& st = states[dev];
+int launch_pair(PairParams& p, float* stats, size_t stats_bytes, cudaStream_t stream) {
+  int rc;
+  const uint32_t clusters = clusters_of<kN>(rc);
+  if (rc != BOOST_OK) return rc;
+  if (clusters == 0) return BOOST_ERR_UNSUPPORTED;
   // activation slots: more than a microsecond of a short product's stream (a k block per 155 ns); from
   // 128 rows on about half of the shared memory, since the tiles are as large as the weight stages
   const uint32_t slot_bytes = x_blocks(kN) * p.nb * 128u;
@@ -1256,76 +1302,54 @@ int launch_pair(PairParams& p, float* stats, size_t stats_bytes, int sms, cudaSt
   p.n_stages = (smem_total(kN) - fixed) / kStageBytes;
   if (p.n_stages > kMaxStages) p.n_stages = kMaxStages;
   const size_t smem = smem_total(kN);
-  if (!st.configured) {
-    int rc = boosth::check(cudaFuncSetAttribute(gemv_pair_kernel<kN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (rc != BOOST_OK) return rc;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2);
-    cfg.blockDim = dim3(threads_of(kN));
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    rc = boosth::check(cudaOccupancyMaxActiveClusters(&n, gemv_pair_kernel<kN>, &cfg));
-    if (rc != BOOST_OK) return rc;
-    st.clusters = (uint32_t)n < (uint32_t)sms / 2 ? (uint32_t)n : (uint32_t)sms / 2;   // one threadblock per SM
-    st.configured = true;
-  }
-  if (st.clusters == 0) return BOOST_ERR_UNSUPPORTED;
   // (the caller's ssq pointers stand in for the buffers until here)
   const float* key[kMaxPhases];
   uint32_t n_stats = 0;
   for (uint32_t i = 0; i < p.n_phases; ++i) {
     PairPhase& q = p.ph[i];
-    plan_phase(q, st.clusters, p.M_b);
+    plan_phase(q, clusters, p.M_b);
     for (int j = (int)i - 1; j >= 0; --j)
       if (q.ssq_in && key[j] == q.ssq_in) {
         q.ssq_in = p.ph[j].ssq_out;
-        q.ssq_parts = ssq_parts_of(p.ph[j], st.clusters);
+        q.ssq_parts = ssq_parts_of(p.ph[j], clusters);
         q.ssq_stride = kN;
         break;
       }
     key[i] = q.ssq_out;
     if (q.ssq_out) {
-      const size_t bytes = (size_t)ssq_parts_of(q, st.clusters) * kN * 4;
+      const size_t bytes = (size_t)ssq_parts_of(q, clusters) * kN * 4;
       if (2 * bytes > stats_bytes) return BOOST_ERR_CAPACITY;
       q.ssq_out = stats + (n_stats++ & 1u) * (stats_bytes / 8);
     }
   }
-  return boosth::launch_chained_cluster(gemv_pair_kernel<kN>, dim3(2 * st.clusters), dim3(threads_of(kN)), smem, 2, stream, p);
+  return boosth::launch_chained_cluster(gemv_pair_kernel<kN>, dim3(2 * clusters), dim3(threads_of(kN)), smem, 2, stream, p);
 }
-
-uint32_t batch_class(uint32_t M_b) { return M_b <= 8 ? 8 : M_b <= 16 ? 16 : M_b <= 32 ? 32 : M_b <= 64 ? 64 : M_b <= 128 ? 128 : 256; }
 
 }  // namespace
 
 size_t boosth::pair_stats_bytes(uint32_t N, uint32_t M_b) {
-  int sms = boosth::sm_count();
-  if (sms <= 0) sms = 148;
-  // two buffers, for whichever way plan_phase cuts the rows
+  // two buffers, for whichever way plan_phase cuts the rows; a workspace may serve smaller batches too
   const uint32_t units = (N + kRowTile - 1) / kRowTile * kUnitsPerTile;
-  return (size_t)2 * sms * images_bound(units, (uint32_t)sms) * 2 * batch_class(M_b) * 4;
+  size_t most = 0;
+  for (uint32_t n = 8; n <= batch_class(M_b); n *= 2) {
+    const uint32_t workers = 2 * clusters_for(n);
+    const size_t bytes = (size_t)2 * workers * images_bound(units, workers) * 2 * n * 4;
+    most = bytes > most ? bytes : most;
+  }
+  return most;
 }
 
-uint32_t boosth::pair_split(uint32_t N, uint32_t K) {
+uint32_t boosth::pair_split(uint32_t N, uint32_t K, uint32_t M_b) {
   PairPhase q = {};
   q.k_blocks = (K + 63) / 64;
   q.n_units = (N + kRowTile - 1) / kRowTile * kUnitsPerTile;
-  const int sms = boosth::sm_count();
-  plan_phase(q, sms > 1 ? (uint32_t)sms / 2 : 1u, 1);
+  plan_phase(q, clusters_for(M_b), M_b);
   return q.split;
 }
 
 int boosth::gemv_pair_launch(const boost_gemv_call_t* calls, uint32_t n_calls, uint32_t M_b, void* workspace, size_t workspace_bytes,
                              uint32_t header_row_tiles, uint32_t* sync_words, bool early, void* stream) {
   if (!calls || n_calls == 0 || n_calls > kMaxPhases || M_b == 0 || M_b > 256) return BOOST_ERR_INVALID;
-  const int sms = boosth::sm_count();
-  if (sms <= 0) return BOOST_ERR_CUDA;
   const size_t header = boosth::gemv_header_bytes(header_row_tiles);
   if (!workspace || workspace_bytes < header) return workspace ? BOOST_ERR_CAPACITY : BOOST_ERR_INVALID;
   float* stats = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + header);
@@ -1383,11 +1407,11 @@ int boosth::gemv_pair_launch(const boost_gemv_call_t* calls, uint32_t n_calls, u
   }
   cudaStream_t st = (cudaStream_t)stream;
   switch (n_class) {
-    case 8: return launch_pair<8>(p, stats, stats_bytes, sms, st);
-    case 16: return launch_pair<16>(p, stats, stats_bytes, sms, st);
-    case 32: return launch_pair<32>(p, stats, stats_bytes, sms, st);
-    case 64: return launch_pair<64>(p, stats, stats_bytes, sms, st);
-    case 128: return launch_pair<128>(p, stats, stats_bytes, sms, st);
-    default: return launch_pair<256>(p, stats, stats_bytes, sms, st);
+    case 8: return launch_pair<8>(p, stats, stats_bytes, st);
+    case 16: return launch_pair<16>(p, stats, stats_bytes, st);
+    case 32: return launch_pair<32>(p, stats, stats_bytes, st);
+    case 64: return launch_pair<64>(p, stats, stats_bytes, st);
+    case 128: return launch_pair<128>(p, stats, stats_bytes, st);
+    default: return launch_pair<256>(p, stats, stats_bytes, st);
   }
 }
