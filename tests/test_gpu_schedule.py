@@ -204,7 +204,7 @@ def test_step_schedule(dev, n_seq, switched):
     finally:
         B.boost_gemv_set_end_combine(True)
     assert torch.equal(dec.buf["logits"][:n_seq], want)                    # logging changes no result
-    recs, _ = check_against_oracle(log, B.SCHED_KIND_GEMV, 64, 1000, 1 / 3)
+    recs, _ = check_against_oracle(log, B.SCHED_KIND_GEMV, 64, 100_000, 1 / 3)
     ly = dec.layers[0]
     for ph, mats in enumerate([(ly["wqkv"], ly["wo"]), (ly["wgu"],), (ly["wd"],), (dec.lm_head,)]):   # (the first product is a launch of its own)
         mine = recs[(recs["kind_phase"] >> 8) == ph]

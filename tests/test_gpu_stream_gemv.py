@@ -178,7 +178,7 @@ def test_gemv_batches(dev, m_b):
     (4096, 14336, 32, 1 / 8),     # down-projection shape: rows of 28 KiB, 57344-byte ... 1.75 pages per row tile
     (6144, 4096, 7, 1 / 3),
     (256, 512, 128, 0.0),
-    (4096, 4096, 256, 1 / 8),     # 256 batch rows: the widest accumulator the tcgen05 kernel takes
+    (4096, 4096, 256, 1 / 8),     # 256 batch rows: the widest accumulator (cluster kernel; two queues: tcgen05 kernel)
 ])
 def test_gemv_shapes(dev, n, k, m_b, ratio):
     w, y, ref, _ = run_gemv(dev, n, k, m_b, ratio, seed=n + k + m_b)
@@ -284,8 +284,9 @@ def test_gemv_tcgen05_and_mma_sync_kernels_agree(dev, m_b):
 @pytest.mark.parametrize("ratio", [0.0, 1 / 64])
 def test_gemv_full_size_batch128(dev, ratio):
     """The gate/up matrix of the bench model (28672 x 4096) at batch 128, the launch of
-    configuration 5 (tcgen05 kernel): all outputs against the oracle; with all pages in HBM
-    (even partition) and with one page in 64 on the host (queue items, host pages first)."""
+    configuration 5 (cluster kernel; with host pages under the two-queue schedule the tcgen05
+    kernel): all outputs against the oracle; with all pages in HBM and with one page in 64 on the
+    host."""
     w, y, ref, _ = run_gemv(dev, 28672, 4096, 128, ratio, seed=21)
     assert w.buf.n_host == (0 if ratio == 0 else w.buf.n_pages // 64)
     # The strict tolerance with the 1e-3 * rms floor, the outputs that miss it counted and held to
@@ -324,3 +325,39 @@ def test_gemv_repeated_launches_are_identical(dev, n, k, m_b, ratio):
         differing += int(not torch.equal(y, first))
     assert differing == 0
     assert w.status_words() == [0]
+
+
+@pytest.mark.parametrize("n,k,m_b", [
+    (1001, 1016, 1), (1001, 1016, 129), (1001, 1024, 1), (1001, 1024, 32), (1001, 1024, 33), (1001, 1024, 129),   # shortest rows of the cluster kernel
+    (1001, 4104, 33), (1001, 8192, 1), (1001, 8192, 256), (1001, 8200, 5),         # longest rows two threadblocks share
+    (9472, 1024, 2), (9473, 1024, 32), (9601, 1024, 3), (9601, 4096, 33), (9473, 4104, 8), (9601, 8192, 2),       # ... and those one has to itself
+    (21, 1024, 17), (128, 1088, 256), (19001, 1032, 65)])
+def test_gemv_at_the_edges_of_the_kernel_rule(dev, n, k, m_b):
+    """Products on both sides of the rule that gives plain products to the cluster kernel, with odd numbers
+    of rows and a residual, in fp32 and bf16, the last page on the host."""
+    tier = np.zeros(B.boost_weight_layout(n, k)["n_pages"], np.uint8)
+    tier[-1] = 1
+    w, y, ref, (x, res) = run_gemv(dev, n, k, m_b, 0.0, seed=n + k + m_b, residual=True, tier=tier)
+    assert_close_to_oracle(y, ref, f"{n} x {k}, batch {m_b}")
+    y16 = w.gemv(x, y_dtype=torch.bfloat16, residual=res).float().cpu().numpy()
+    # A bf16 rounding (at most 2^-8 of the value) of sums whose accumulators hold up to 4096 columns: 256
+    # additions that truncate by at most 2^-23 of what the accumulator holds, which is rarely more than twice the rms.
+    assert (np.abs(y16 - y) <= np.abs(y) * 2.0 ** -8 + 2 * 256 * 2.0 ** -23 * np.sqrt((ref * ref).mean())).all()
+    assert w.status_words() == [0]
+
+
+@pytest.mark.parametrize("n,k,m_b", [(28672, 4096, 64), (4096, 4096, 256), (4096, 4096, 24), (6144, 4096, 7)])
+def test_split_k_kernels_at_full_size(dev, n, k, m_b):
+    """The kernels whose partial sums meet in L2 at the sizes that plain products now take to the cluster kernel:
+    a switch at another value than its default brings them back (64 and 256 rows: tcgen05, fewer: mma.sync)."""
+    try:
+        B.boost_gemv_set_tc_min_batch(34)
+        w, y, ref, _ = run_gemv(dev, n, k, m_b, 1 / 16, seed=3)
+        # (28672 x 4096: a handful of 1.8 million outputs next to zero miss the relative bound, see
+        # test_gemv_full_size_batch128; their absolute error is what 256 truncating additions leave)
+        n_floor, exceptions = assert_close_to_oracle(y, ref, f"{n} x {k}, batch {m_b}", report_exceptions=True)
+        rms = float(np.sqrt((ref * ref).mean()))
+        assert len(exceptions) <= 16 and all(abs(r) < 2e-3 * rms and e <= 4 * 256 * 2.0 ** -24 * rms for r, e in exceptions)
+        assert w.status_words() == [0]
+    finally:
+        B.boost_gemv_set_tc_min_batch(33)
