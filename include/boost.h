@@ -382,8 +382,9 @@ int boost_pack_weights_ex(const void* w_row_major /*device*/, uint32_t N, uint32
  * Everything is read after the kernels ahead of the call on the stream have finished: pages and page
  * tables may have been written there.  (So has everything ahead of a decode step when its first
  * product starts; after that a step reads weights while its own kernels run, none of which writes them.)
- * Products with rows of 1024 to 4096 columns (8192 where few rows leave two threadblocks to share
- * each) run on tcgen05 cut along the rows of the weight, in one launch without partial sums in memory.
+ * Most products with rows of 1024 to 4096 columns (8192 where few rows leave two threadblocks to share
+ * each) run on tcgen05 cut along the rows of the weight, in one launch without partial sums in memory;
+ * few long rows, and others that would take longer there, do not.
  * Of the others, M_b <= 2 runs on CUDA cores with warp-shuffle reductions; larger batches use the
  * tensor cores (mma.sync up to 32 rows, tcgen05 with accumulators in tensor memory above; see
  * boost_gemv_set_tc_min_batch).  There the blocks of a weight are cut evenly over the threadblocks;

@@ -101,8 +101,10 @@ int encode_activation_map(void* map, const void* x, uint32_t M_b, uint32_t K, ui
 size_t pair_stats_bytes(uint32_t N, uint32_t M_b);
 int gemv_pair_launch(const boost_gemv_call_t* calls, uint32_t n_calls, uint32_t M_b, void* workspace, size_t workspace_bytes,
                      uint32_t header_row_tiles, uint32_t* sync_words, bool early, void* stream);
-// How many threadblocks of a cluster share the columns of a product there (1 or 2).
-uint32_t pair_split(uint32_t N, uint32_t K, uint32_t M_b);
+// How a product is cut there: threadblocks, how many of a cluster share its columns (1 or 2), and the units of
+// 4 + 4 rows of the widest worker.
+struct PairCut { uint32_t threadblocks, split, units; };
+PairCut pair_cut(uint32_t N, uint32_t K, uint32_t M_b);
 // The argument checks every weight product goes through.
 int gemv_check_call(const boost_gemv_call_t& call, uint32_t M_b, void* workspace, size_t workspace_bytes, uint32_t header_row_tiles);
 // Whether the process-wide switches leave products (with host pages or without) to the cluster kernel.

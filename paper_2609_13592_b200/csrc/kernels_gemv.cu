@@ -1970,9 +1970,38 @@ int boosth::gemv_chain_launch(const boost_gemv_call_t* calls, uint32_t n_calls, 
 //     are not measured on it (in a step they are: the down product's 7168);
 //   - the rows are short: a threadblock's time is then its epilogue, and the kernels above finish
 //     tiles from tensor memory;
+//   - the product would take longer there (cluster_faster below);
 //   - y overlaps x: a threadblock writes its rows while others still read x;
 //   - one of the process-wide switches that choose among the kernels above is not at its default.
 constexpr uint32_t kPairMaxDepth = 4096, kPairMinColumns = 1024;
+
+// Microseconds of a product on its own, fitted to 19 numbers of rows (130 - 30000) x 8 lengths (1024 - 8192) x 13
+// batches x fp32 / bf16 results.  Cluster kernel: a threadblock goes through its share of the columns
+// k block by k block, each as long as its instructions and activations (longer for fp32 results, whose
+// accumulators are short) and its rows' weights; split-K kernels: the threadblock's share of all
+// blocks, and the partial sums of a row tile.  So few long rows are better off cut finely (1000 x 8192: 15 us against 17 at
+// batch 1, 24 against 52 at 256 and fp32), and so are rows just too many to be shared (10000 x 4096, batch 1: 1.17 x).
+// The better of the two is taken within 0.5 % on average; always the cluster kernel 8.8 %, never 15 %.
+struct ProductCost {
+  float fixed, block, block_fp32, unit;        // cluster kernel
+  float split_fixed, split_block, split_sums;  // split-K kernels
+};
+constexpr ProductCost kProductCost[6][2] = {   // batches up to 8, 16, 32, 64, 128, 256; columns shared by two threadblocks, or not
+    {{4.968f, 0.112f, 0.026f, 0.007f, 6.714f, 0.333f, 0.115f}, {5.344f, 0.045f, 0.017f, 0.020f, 10.813f, 0.332f, -2.164f}},
+    {{5.250f, 0.118f, 0.040f, 0.006f, 7.038f, 0.327f, 0.117f}, {5.705f, 0.038f, 0.016f, 0.020f, 11.541f, 0.327f, -2.444f}},
+    {{5.735f, 0.141f, 0.055f, 0.003f, 7.770f, 0.421f, 0.127f}, {6.323f, 0.034f, 0.012f, 0.022f, 14.946f, 0.376f, -3.407f}},
+    {{7.448f, 0.150f, 0.069f, 0.003f, 9.076f, 0.422f, 0.078f}, {7.207f, 0.030f, 0.011f, 0.023f, 13.157f, 0.403f, -1.842f}},
+    {{8.160f, 0.228f, 0.125f, -0.001f, 10.40f, 0.616f, 0.057f}, {8.822f, 0.042f, 0.013f, 0.027f, 20.174f, 0.463f, -3.504f}},
+    {{11.30f, 0.261f, 0.165f, -0.006f, 12.04f, 0.879f, 0.051f}, {10.366f, 0.015f, 0.019f, 0.035f, 29.06f, 0.666f, -6.498f}}};
+
+static bool cluster_faster(uint32_t N, uint32_t K, uint32_t M_b, bool fp32, const boosth::PairCut& cut) {
+  const uint32_t batch = M_b <= 8 ? 0 : M_b <= 16 ? 1 : M_b <= 32 ? 2 : M_b <= 64 ? 3 : M_b <= 128 ? 4 : 5;
+  const ProductCost& c = kProductCost[batch][cut.split == 2 ? 0 : 1];
+  const float tiles = (float)((N + kBlockRows - 1) / kBlockRows), k_blocks = (float)((K + kBlockK - 1) / kBlockK);
+  const float own = k_blocks / (float)cut.split, per_tile = (float)cut.threadblocks / tiles;
+  return c.fixed + own * (c.block + (fp32 ? c.block_fp32 : 0.f) + c.unit * (float)cut.units) <=
+         c.split_fixed + c.split_block * tiles * k_blocks / (float)cut.threadblocks + c.split_sums * (per_tile < k_blocks ? per_tile : k_blocks);
+}
 
 bool boosth::cluster_products(bool host_pages) {
   return g_tc_min_batch == kTcMinBatchDefault && g_end_combine && !(g_tier_schedule && host_pages);
@@ -1981,7 +2010,8 @@ bool boosth::cluster_products(bool host_pages) {
 static bool cluster_takes(const boost_gemv_call_t& c, uint32_t M_b) {
   if (c.has_epilogue && (c.epilogue.mode != BOOST_EPI_PLAIN || c.epilogue.ssq_in || c.epilogue.ssq_out)) return false;
   if (c.w.N == 0 || c.w.K < kPairMinColumns || !boosth::cluster_products(c.w.n_host_pages != 0)) return false;
-  if (c.w.K > kPairMaxDepth * boosth::pair_split(c.w.N, c.w.K, M_b)) return false;
+  const boosth::PairCut cut = boosth::pair_cut(c.w.N, c.w.K, M_b);
+  if (c.w.K > kPairMaxDepth * cut.split || !cluster_faster(c.w.N, c.w.K, M_b, c.y_dtype == 0, cut)) return false;
   const uint8_t *x = static_cast<const uint8_t*>(c.x), *y = static_cast<const uint8_t*>(c.y);
   const size_t x_bytes = (size_t)M_b * c.w.K * 2, y_bytes = (size_t)M_b * c.w.N * (c.y_dtype == 0 ? 4 : 2);
   return x + x_bytes <= y || y + y_bytes <= x;

@@ -1339,12 +1339,13 @@ size_t boosth::pair_stats_bytes(uint32_t N, uint32_t M_b) {
   return most;
 }
 
-uint32_t boosth::pair_split(uint32_t N, uint32_t K, uint32_t M_b) {
+boosth::PairCut boosth::pair_cut(uint32_t N, uint32_t K, uint32_t M_b) {
   PairPhase q = {};
   q.k_blocks = (K + 63) / 64;
   q.n_units = (N + kRowTile - 1) / kRowTile * kUnitsPerTile;
-  plan_phase(q, clusters_for(M_b), M_b);
-  return q.split;
+  const uint32_t clusters = clusters_for(M_b);
+  plan_phase(q, clusters, M_b);
+  return {2 * clusters, q.split, units_bound(q.n_units, q.split == 2 ? clusters : 2 * clusters)};
 }
 
 int boosth::gemv_pair_launch(const boost_gemv_call_t* calls, uint32_t n_calls, uint32_t M_b, void* workspace, size_t workspace_bytes,

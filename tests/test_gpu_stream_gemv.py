@@ -361,3 +361,38 @@ def test_split_k_kernels_at_full_size(dev, n, k, m_b):
         assert w.status_words() == [0]
     finally:
         B.boost_gemv_set_tc_min_batch(33)
+
+
+@pytest.mark.parametrize("n,k,m_b", [(1000, 8192, 1), (1000, 8192, 256), (10000, 4096, 1), (500, 4096, 200), (300, 8192, 64)])
+def test_products_that_are_better_off_split_finely(dev, n, k, m_b):
+    """Few long rows, and rows just too many for two threadblocks to share, take the kernels whose partial sums
+    meet in memory: against the oracle, and no slower than under the switch that asks for them (a tenth
+    for the clock; on the cluster kernel they were 1.15 to 2.6 times slower)."""
+    from paper_2609_13592_b200.tiers import TieredWeight
+    w, y, ref, (x, _) = run_gemv(dev, n, k, m_b, 0.0, seed=n + m_b)
+    assert_close_to_oracle(y, ref, f"{n} x {k}, batch {m_b}")
+    out = torch.empty(m_b, n, device=dev)
+    graphs = []
+    try:
+        for threshold in (33, 34):
+            B.boost_gemv_set_tc_min_batch(threshold)
+            w.gemv(x, y=out)
+            torch.cuda.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                for _ in range(20):
+                    w.gemv(x, y=out)
+            graphs.append(g)
+    finally:
+        B.boost_gemv_set_tc_min_batch(33)
+    times = [[], []]
+    for _ in range(7):
+        for g, t in zip(graphs, times):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            g.replay()
+            b.record()
+            torch.cuda.synchronize()
+            t.append(a.elapsed_time(b))
+    assert min(times[0]) <= 1.1 * min(times[1])
+    assert w.status_words() == [0]
