@@ -637,7 +637,9 @@ typedef struct {
 
 /* Device scratch of a decode step for up to ssq_stride sequences (bf16 unless noted):
  * h [B, hidden] (residual stream); q_rot, attn [B, Hq D]; act [B, F]; logits fp32 [B, vocab];
- * ssq_a, ssq_b fp32 [hidden / 128][ssq_stride] (row statistics for the RMS scales); rope_table
+ * ssq_a, ssq_b fp32 [hidden / 128][ssq_stride] (row statistics for the RMS scales: ssq_a of the embedded
+ * tokens; later ones pass from product to product in gemv_ws, or through both under a switch that
+ * brings the split-K kernels back); rope_table
  * fp32 [B][64][2];
  * gemv_ws >= boost_llama_gemv_workspace_bytes(model, B) (counters sized for the widest
  * product, the largest set of partial sums, one set of queue words per launch); attn_ws >=

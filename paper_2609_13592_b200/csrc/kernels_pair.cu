@@ -93,8 +93,8 @@ struct PairParams {
 };
 
 // kN: the batch class of an instantiation (8, 16, 32, 64, 128, 256 rows).
-// Activations by tiled TMA copies, or by one warp's 16-byte copies (3-layer step, 16-byte copies against
-// TMA: batch 1 465 / 473 us, 8 500 / 506, 32 636 / 641; more rows are too many copies for one warp).
+// Activations by tiled TMA copies, or by one warp's 16-byte copies (measured when both were built: TMA 1.7 % slower
+// for a step at batch 1, 1.2 % at 8, 0.8 % at 32; more rows are too many copies for one warp).
 __host__ __device__ constexpr bool x_by_tma(uint32_t n) { return n > 32; }
 // k blocks of an activation slot.  (Up to 16 rows four: half the barrier polls and commits of the MMA warp.)
 __host__ __device__ constexpr uint32_t x_blocks(uint32_t n) { return n <= 16 ? 4 : n >= 128 ? 1 : 2; }
@@ -121,7 +121,7 @@ __host__ __device__ constexpr uint32_t epi_warps(uint32_t n) { return n <= 32 ? 
 __host__ __device__ constexpr uint32_t threads_of(uint32_t n) { return (kEpiWarp0 + epi_warps(n)) * 32; }
 // Sums on their way from tensor memory to the threads that finish them, fp32 [columns][128 lanes].
 // Rows of one threadblock: this many columns at a time (from 64 rows on 64 in one buffer; 32 in two
-// buffers in turn: 3-layer step at batch 128 1150 us either way, at batch 250 1257 against 1238).
+// buffers in turn were the same at batch 128 and 1.5 % slower for a step at batch 250).
 __host__ __device__ constexpr uint32_t chunk_cols(uint32_t n) { return n < 64 ? n : 64; }
 // Rows that two threadblocks share: each finishes half of the columns, in this many rounds.  The
 // columns of a round, this threadblock's sums and the peer's, are kept in the chunk buffers
@@ -1232,8 +1232,8 @@ uint32_t ssq_parts_of(const PairPhase& q, uint32_t clusters) { return (q.split =
 
 // Shared memory of an instantiation.  More than half an SM, so that no two threadblocks of this kernel
 // share one (the grid counts on one threadblock per SM).  Up to 32 rows a threadblock of the
-// attention kernel fits beside it (measured, 3-layer step at batch 1 / 32: 493 / 683 us with 145 KiB,
-// 507 / 685 with 180); above, the activation tiles need the room.
+// attention kernel fits beside it (measured when it was chosen: a step at batch 1 is 2.8 % slower with
+// 180 KiB, at batch 32 0.3 %); above, the activation tiles need the room.
 constexpr uint32_t smem_total(uint32_t n) { return (n <= 32 ? 147u : 214u) * 1024u; }
 
 // Clusters of two that the current device holds at once, one threadblock per SM (0: none, or an error, which
