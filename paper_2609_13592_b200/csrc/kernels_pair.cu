@@ -23,17 +23,17 @@
 // activation tiles side by side took fewer MMAs and the same time, but half of its results were
 // nobody's: at batch 32 the GPU is at its power limit, and a step of 4690 us became one of 4640.)
 //
-// One threadblock per SM.  Up to 32 batch rows it takes 147 KiB of shared memory and 96 registers per
+// One threadblock per SM.  Up to 32 batch rows it takes 147 KiB of shared memory and 80 registers per
 // thread: a threadblock of the attention kernel before and after it on the stream fits beside it, and
 // the weights of the first product are in place when the kernel before it ends.  A ring of 64 KiB
 // per SM already saturates HBM (measured with bulk copies of 2 - 16 KiB: 48 KiB 6.3, 64 KiB 6.8, 80
 // - 112 KiB 6.9, 192 KiB 6.4 - 6.7 TB/s), so sharing the SM costs no bandwidth.  Larger batches take
 // the whole SM: their activation tiles are up to 32 KiB each.
 //
-// Warps: 0 and 3 weight producers (every other stage each: one warp's instruction latency would bound
-// the stream of a product whose stages are four or eight copies), 1 activation producer, 2 MMA
-// issue and tensor-memory allocation, 4 and up epilogue.  The first four run warp-uniform code and
-// elect a lane for the copy or MMA itself: inside an if (lane == 0) every operand goes through a
+// Warps: 0 and 3 weight producers (a pipeline each, or every other stage: one warp's instruction latency
+// would bound the stream of a product whose stages are four or eight copies), 1 activation producer, 2 MMA
+// issue and tensor-memory allocation, 4 and up epilogue, the last one (up to 128 rows) the second pipeline's
+// MMA issue.  Producers and MMA warps run warp-uniform code and elect a lane for the copy or MMA itself: inside an if (lane == 0) every operand goes through a
 // vector register (measured: a group of four MMAs and a commit 293 cycles against 212, a bulk copy 64
 // against 25).
 #include <cuda.h>
@@ -53,7 +53,7 @@ constexpr uint32_t kRowTile = 128;
 constexpr uint32_t kBlockBytes = 16384;                        // 128 rows x 64 columns of bf16
 constexpr uint32_t kBlocksPerPage = kPageBytes / kBlockBytes;  // 128
 constexpr uint32_t kUnitsPerTile = 16;                         // units of 4 + 4 rows
-constexpr uint32_t kEpiWarp0 = 4;                              // warps 0 - 3: producers and MMA issue
+constexpr uint32_t kEpiWarp0 = 4;                              // warps 0 - 3: producers, the first MMA warp; then epilogue, the second MMA warp
 constexpr uint32_t kStageBytes = kBlockBytes;                  // one image of 16 units, or two k blocks of an image of 8
 constexpr uint32_t kMaxStages = 12, kMaxXSlots = 12;
 constexpr uint32_t kMaxPhases = 4;
@@ -67,7 +67,8 @@ struct PairPhase {
   uint32_t split;            // 2: the cluster's threadblocks take half of K each; 1: every threadblock has rows of its own
   uint32_t image;            // units of an image: 16, or 8 where no worker has more (then a stage holds two k blocks)
   uint32_t max_images;       // images of the widest worker
-  uint32_t part_blocks;      // k blocks of an accumulator; 0: a quarter of a block
+  uint32_t mode;             // an accumulator holds a quarter of a k block (0), a k block (1), several (2)
+  uint32_t slot_blocks;      // k blocks of a slot of accumulators
   void* y;
   int y_dtype;
   const __nv_bfloat16* residual;
@@ -96,33 +97,39 @@ struct PairParams {
 // Activations by tiled TMA copies, or by one warp's 16-byte copies (measured when both were built: TMA 1.7 % slower
 // for a step at batch 1, 1.2 % at 8, 0.8 % at 32; more rows are too many copies for one warp).
 __host__ __device__ constexpr bool x_by_tma(uint32_t n) { return n > 32; }
-// k blocks of an activation slot.  (Up to 16 rows four: half the barrier polls and commits of the MMA warp.)
-__host__ __device__ constexpr uint32_t x_blocks(uint32_t n) { return n <= 16 ? 4 : n >= 128 ? 1 : 2; }
+// k blocks of an activation slot.
+__host__ __device__ constexpr uint32_t x_blocks(uint32_t n) { return n >= 128 ? 1 : 2; }
 // The tensor cores' fp32 adder truncates: every MMA that adds to an accumulator takes about 2.7e-8 of
 // what it holds, always towards zero, so a sum over n MMAs is off by n / 2 times that (2-norm against
 // fp64, normal inputs, 32 / 128 / 256 MMAs: 4.5e-7, 2.1e-6, 4.4e-6).  An accumulator therefore holds a PART
-// of the columns only (PairPhase::part_blocks), and the epilogue warps take the parts out of tensor
+// of the columns only (plan_parts), and the epilogue warps take the parts out of tensor
 // memory as they come and add them up where additions round to nearest.
 // Parts of part_cols columns (an M = 128 product has at least 16) change hands in slots of up to
 // slot_parts; as many slots as tensor memory holds are in flight.
+// Up to 128 rows there are two pipelines (a weight producer, a ring of stages and one of activation slots, an MMA
+// warp and accumulators each), which take the chunks of a slot's k blocks in turn: a part that holds several
+// blocks has every other chunk.  At 256 rows there is one: its MMAs take longer than what the issuing
+// warp does between them, and tensor memory holds two accumulators only.
+__host__ __device__ constexpr uint32_t pipes_of(uint32_t n) { return n <= 128 ? 2 : 1; }
 __host__ __device__ constexpr uint32_t part_cols(uint32_t n) { return n < 16 ? 16 : n; }
-__host__ __device__ constexpr uint32_t slot_parts(uint32_t n) { return n <= 8 ? 16 : n <= 16 ? 4 : n <= 64 ? 2 : 1; }
+__host__ __device__ constexpr uint32_t slot_parts(uint32_t n) { return n <= 8 ? 16 : n <= 64 ? 4 : n <= 128 ? 2 : 1; }
 __host__ __device__ constexpr uint32_t slot_cols(uint32_t n) { return part_cols(n) * slot_parts(n); }
 constexpr uint32_t kMaxAccSlots = 8;
 __host__ __device__ constexpr uint32_t acc_slots(uint32_t n) { return 512 / slot_cols(n) < kMaxAccSlots ? 512 / slot_cols(n) : kMaxAccSlots; }
 __host__ __device__ constexpr uint32_t tmem_cols(uint32_t n) { return acc_slots(n) * slot_cols(n); }
-// k blocks of a slot whose parts are part_blocks (0: a quarter of a block, one MMA) each.
-__host__ __device__ constexpr uint32_t slot_blocks(uint32_t n, uint32_t part_blocks) {
-  return part_blocks == 0 ? slot_parts(n) / 4 : part_blocks == 1 ? slot_parts(n) : part_blocks;
+// k blocks of a chunk.  (A slot holds a multiple of that, but at the end of K.)
+__host__ __device__ constexpr uint32_t chunk_blocks(uint32_t n, uint32_t image) {
+  return pipes_of(n) == 1 ? 1 : image == 8 || x_blocks(n) == 2 ? 2 : 1;
 }
 // Epilogue warps: a short product's last accumulator is finished by all of them at the end of a phase,
 // which at large batches is bound by their instruction latency.
 __host__ __device__ constexpr uint32_t epi_warps(uint32_t n) { return n <= 32 ? 8 : 16; }
-__host__ __device__ constexpr uint32_t threads_of(uint32_t n) { return (kEpiWarp0 + epi_warps(n)) * 32; }
+__host__ __device__ constexpr uint32_t threads_of(uint32_t n) { return (kEpiWarp0 + epi_warps(n) + pipes_of(n) - 1) * 32; }
 // Sums on their way from tensor memory to the threads that finish them, fp32 [columns][128 lanes].
-// Rows of one threadblock: this many columns at a time (from 64 rows on 64 in one buffer; 32 in two
-// buffers in turn were the same at batch 128 and 1.5 % slower for a step at batch 250).
-__host__ __device__ constexpr uint32_t chunk_cols(uint32_t n) { return n < 64 ? n : 64; }
+// Rows of one threadblock: this many columns at a time (32 in two buffers in turn were 1.5 % slower than 64
+// for a step at batch 250).  128 rows: 32, so that shared memory holds six stages and six activation slots
+// (6-layer step at batch 128: 1503 us; 64 columns with six stages and four slots 1584, with four and six 1605).
+__host__ __device__ constexpr uint32_t chunk_cols(uint32_t n) { return n < 64 ? n : n == 128 ? 32 : 64; }
 // Rows that two threadblocks share: each finishes half of the columns, in this many rounds.  The
 // columns of a round, this threadblock's sums and the peer's, are kept in the chunk buffers
 // (up to 32 rows) or in the activation slots, which are idle then.
@@ -298,8 +305,8 @@ __device__ __noinline__ uint32_t host_bytes_of_range(const PairPhase& q, uint32_
 }
 
 template <uint32_t kN>
-__global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairParams p) {
-  constexpr uint32_t kXB = x_blocks(kN), kSlots = acc_slots(kN), kSlotCols = slot_cols(kN);
+__global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_constant__ PairParams p) {
+  constexpr uint32_t kXB = x_blocks(kN), kSlots = acc_slots(kN), kSlotCols = slot_cols(kN), kPipes = pipes_of(kN);
   constexpr bool kTmaX = x_by_tma(kN);
   constexpr uint32_t kEpiWarps = epi_warps(kN), kEpiThreads = kEpiWarps * 32;
   constexpr bool kBig = kN >= 64;
@@ -313,7 +320,7 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
   // (an 8-row activation tile is read as 16 rows: 1 KiB behind the slots)
   float* sums = reinterpret_cast<float*>(x_ring + x_slot * x_slots + 1024u);
   __shared__ uint64_t w_full[kMaxStages], w_empty[kMaxStages], x_full[kMaxXSlots], x_empty[kMaxXSlots];
-  __shared__ uint64_t acc_full[kMaxAccSlots], acc_empty[kMaxAccSlots], xch_full, xch_free, go, drained;
+  __shared__ uint64_t acc_full[kMaxAccSlots], acc_empty[kMaxAccSlots], xch_full, xch_free, go, drained[2];
   __shared__ uint32_t s_tmem;
   __shared__ uint32_t s_rec[kMaxPhases];
   __shared__ float s_rs[kN], s_red[kEpiThreads];
@@ -332,13 +339,14 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
     for (uint32_t s = 0; s < n_stages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); }
     for (uint32_t s = 0; s < x_slots; ++s) { mbar_init(&x_full[s], kTmaX ? 1 : 32); mbar_init(&x_empty[s], 1); }
     for (uint32_t s = 0; s < kSlots; ++s) {
-      mbar_init(&acc_full[s], 1);
+      mbar_init(&acc_full[s], kPipes);
       mbar_init(&acc_empty[s], kEpiWarps);
     }
     mbar_init(&xch_full, 1);
     mbar_init(&xch_free, 1);
     mbar_init(&go, 1);
-    mbar_init(&drained, 1);
+    mbar_init(&drained[0], 1);
+    mbar_init(&drained[1], 1);
     s_abort = 0;
     fence_barrier_init();
   }
@@ -364,25 +372,32 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
     r.kb1 = two ? q.k_blocks * (rank + 1) / 2 : q.k_blocks;
     return r;
   };
+  // A pipeline's stages (activation slots) are behind each other.
+  const uint32_t pipe_stages = n_stages / kPipes, pipe_slots = x_slots / kPipes;
   // Where a producer warp stands: the stage (activation slot) it would fill next, the parity of its wait for
-  // it, and whether it is this warp's turn.  Known at the end of the kernel too, for the wind-down.
+  // it (the activation producer's second pipeline: stage1, parity1), and whether it is this warp's turn.
+  // Known at the end of the kernel too, for the wind-down.
   uint32_t stage = 0, parity = 1;
-  bool my_turn = warp != 3;
+  [[maybe_unused]] uint32_t stage1 = 0, parity1 = 1;
+  bool my_turn = kPipes == 2 || warp != 3;
 
   if (warp == 0 || warp == 3) {
     // ------------------------------------------------------------------ weight producers
-    const uint32_t ring_a = smem_u32(ring), full_a = smem_u32(w_full), empty_a = smem_u32(w_empty);
+    const uint32_t pipe = kPipes == 2 && warp == 3 ? 1u : 0u, first = pipe * pipe_stages;
+    const uint32_t ring_a = smem_u32(ring) + first * kStageBytes, full_a = smem_u32(w_full) + first * 8, empty_a = smem_u32(w_empty) + first * 8;
     if (!p.early) {
       pdl_wait();
       fence_proxy_async_all();   // pages written with ordinary stores are read through the TMA unit
     }
     unsigned long long* const log = sched_log_of(p.ws);
+    // Two pipelines: each of the two warps has one.  One: they take its stages in turn.
     // Per stage: wait, announce the bytes, copy.  Everything else is kept out of the loop: the lanes
     // hold the pieces' addresses (part of the run x lower / upper rows; x k block of an image of 8), and
     // step through K on their own.
     auto produce = [&](const PairPhase& q, uint32_t ph) -> bool {
       const Part w = part_of(q);
       const uint32_t image = q.image, k_blocks = q.k_blocks, n_pages = q.n_pages;
+      [[maybe_unused]] const uint32_t slot_n = q.slot_blocks, chunk = chunk_blocks(kN, image);
       const void* const* const page_ptr = q.w_page_ptr;
       const bool twos = image == 8;
       if (warp == 0 && lane == 0) {
@@ -407,35 +422,42 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
         }
         const uint32_t to = ring_a + second * (kStageBytes / 2) + half * image * 512u + (a % image) * 512u;
         const uint32_t in_block = (half * 64u + (a % kUnitsPerTile) * 4u) * 128u;
-        uint32_t blk = a / kUnitsPerTile * k_blocks + w.kb0 + second, page = 0xFFFFFFFFu;
-        const uint8_t *src = nullptr, *next = nullptr;   // the next block of this piece; the page after its page
-        auto locate = [&]() {   // (at the start, and where K runs into another page)
-          const uint32_t pg = blk / kBlocksPerPage;
-          const uint8_t* base = pg == page + 1 && next ? next : static_cast<const uint8_t*>(page_ptr[pg]);
-          page = pg;
-          next = pg + 1 < n_pages ? static_cast<const uint8_t*>(page_ptr[pg + 1]) : nullptr;
-          src = base + (size_t)(blk % kBlocksPerPage) * kBlockBytes + in_block;
-        };
-        if (mine && w.kb0 + second < w.kb1) locate();
+        const uint32_t tile = a / kUnitsPerTile * k_blocks;   // the row tile's first block
+        uint32_t page = 0xFFFFFFFFu;
+        const uint8_t *base = nullptr, *next = nullptr;   // the page of this piece's block, and the one after it
         const uint32_t tx = (ub - ua) * 1024u * step;
-        for (uint32_t kb = w.kb0; kb < w.kb1; kb += step) {
-          if (mine && second && kb + 1 == w.kb1) {
-            // an odd last block is its own partner (it meets zeros, or nothing)
-            const uint32_t b0 = blk - 1;
-            src = static_cast<const uint8_t*>(page_ptr[b0 / kBlocksPerPage]) + (size_t)(b0 % kBlocksPerPage) * kBlockBytes + in_block;
+        auto fill = [&](uint32_t kb) -> bool {   // the next stage: block kb (and the next of an image of 8; an odd last one is its own partner: it meets zeros, or nothing)
+          if (!wait(empty_a + stage * 8, parity)) return false;
+          const uint32_t full = full_a + stage * 8;
+          if (lane == 0) expect_tx(full, tx);
+          __syncwarp();
+          if (mine) {
+            const uint32_t blk = tile + min(kb + second, w.kb1 - 1), pg = blk / kBlocksPerPage;
+            if (pg != page) {   // (at the start, and where K runs into another page)
+              base = pg == page + 1 && next ? next : static_cast<const uint8_t*>(page_ptr[pg]);
+              page = pg;
+              next = pg + 1 < n_pages ? static_cast<const uint8_t*>(page_ptr[pg + 1]) : nullptr;
+            }
+            bulk_copy(to + stage * kStageBytes, base + (size_t)(blk % kBlocksPerPage) * kBlockBytes + in_block, bytes, full);
           }
-          if (my_turn) {
-            if (!wait(empty_a + stage * 8, parity)) return false;
-            const uint32_t full = full_a + stage * 8;
-            if (lane == 0) expect_tx(full, tx);
-            __syncwarp();
-            if (mine) bulk_copy(to + stage * kStageBytes, src, bytes, full);
+          return true;
+        };
+        auto next_stage = [&]() { if (++stage == pipe_stages) { stage = 0; parity ^= 1u; } };
+        if constexpr (kPipes == 2) {
+          for (uint32_t k0 = w.kb0; k0 < w.kb1; k0 += slot_n) {
+            const uint32_t k1 = min(k0 + slot_n, w.kb1);
+            for (uint32_t kb = k0 + pipe * chunk; kb < k1; kb += 2 * chunk)
+              for (uint32_t j = kb; j < min(kb + chunk, k1); j += step) {
+                if (!fill(j)) return false;
+                next_stage();
+              }
           }
-          my_turn = !my_turn;
-          if (++stage == n_stages) { stage = 0; parity ^= 1u; }
-          blk += step;
-          src += step * kBlockBytes;
-          if (mine && blk % kBlocksPerPage < step && kb + step + second < w.kb1) locate();
+        } else {
+          for (uint32_t kb = w.kb0; kb < w.kb1; kb += step) {
+            if (my_turn && !fill(kb)) return false;
+            my_turn = !my_turn;
+            next_stage();
+          }
         }
       }
       return true;
@@ -454,59 +476,82 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
       __syncwarp();
     }
     pdl_wait();
-    uint32_t& xs = stage;
+    // fill(kb, slot, parity): the k blocks of a slot from kb on.  For every slot of a phase, the pipelines' chunks in turn.
+    auto in_order = [&](const PairPhase& q, const Part& w, auto fill) -> bool {
+      [[maybe_unused]] const uint32_t slot_n = q.slot_blocks, chunk = chunk_blocks(kN, q.image);
+      for (uint32_t pa = w.u0; pa < w.u1; pa += w.run) {
+        if constexpr (kPipes == 1) {
+          for (uint32_t kb = w.kb0; kb < w.kb1; kb += kXB) {
+            if (!fill(kb, stage, parity)) return false;
+            if (++stage == pipe_slots) { stage = 0; parity ^= 1u; }
+          }
+        } else {
+          for (uint32_t k0 = w.kb0; k0 < w.kb1; k0 += slot_n) {
+            const uint32_t k1 = min(k0 + slot_n, w.kb1);
+            for (uint32_t c = k0; c < k1; c += 2 * chunk) {
+              for (uint32_t kb = c; kb < min(c + chunk, k1); kb += kXB) {
+                if (!fill(kb, stage, parity)) return false;
+                if (++stage == pipe_slots) { stage = 0; parity ^= 1u; }
+              }
+              for (uint32_t kb = c + chunk; kb < min(c + 2 * chunk, k1); kb += kXB) {
+                if (!fill(kb, pipe_slots + stage1, parity1)) return false;
+                if (++stage1 == pipe_slots) { stage1 = 0; parity1 ^= 1u; }
+              }
+            }
+          }
+        }
+      }
+      return true;
+    };
     auto produce = [&](const PairPhase& q, uint32_t ph) -> bool {
       const Part w = part_of(q);
-      const uint32_t K = q.K, run = w.run;
+      const uint32_t K = q.K;
       if constexpr (kTmaX) {
         fence_proxy_async_all();   // x was written with ordinary stores and is read through the TMA unit
-        for (uint32_t pa = w.u0; pa < w.u1; pa += run)
-          for (uint32_t kb = w.kb0; kb < w.kb1; kb += kXB) {
-            if (!wait(empty_a + xs * 8, parity)) return false;
-            if (elect_one()) {
-              const uint32_t full = full_a + xs * 8, dst = x_a + xs * x_slot;
-              expect_tx(full, x_slot);
-              tma_tile(dst, &p.x_map[ph], (int32_t)(kb * 64u), full);
-              // (behind an odd last block: columns outside the tensor, which arrive as zeros)
-              if constexpr (kXB == 2) tma_tile(dst + x_block, &p.x_map[ph], (int32_t)((kb + 1 < w.kb1 ? kb + 1 : q.k_blocks) * 64u), full);
-            }
-            __syncwarp();
-            if (++xs == x_slots) { xs = 0; parity ^= 1u; }
+        return in_order(q, w, [&](uint32_t kb, uint32_t xs, uint32_t par) -> bool {
+          if (!wait(empty_a + xs * 8, par)) return false;
+          if (elect_one()) {
+            const uint32_t full = full_a + xs * 8, dst = x_a + xs * x_slot;
+            expect_tx(full, x_slot);
+            tma_tile(dst, &p.x_map[ph], (int32_t)(kb * 64u), full);
+            // (behind an odd last block: columns outside the tensor, which arrive as zeros)
+            if constexpr (kXB == 2) tma_tile(dst + x_block, &p.x_map[ph], (int32_t)((kb + 1 < w.kb1 ? kb + 1 : q.k_blocks) * 64u), full);
           }
+          __syncwarp();
+          return true;
+        });
       } else {
         const uint32_t c = lane & 7, r0 = lane >> 3, M_b = p.M_b;
         const uint32_t to0 = x_a + r0 * 128u + ((c ^ r0) << 4), to1 = x_a + (r0 + 4) * 128u + ((c ^ (r0 + 4)) << 4);   // rows 8 i + r0, 8 i + 4 + r0
         const __nv_bfloat16* const x0 = q.x + (size_t)r0 * K + (c * 8u < K ? c * 8u : 0u);
-        for (uint32_t pa = w.u0; pa < w.u1; pa += run)
-          for (uint32_t kb = w.kb0; kb < w.kb1; kb += kXB) {
-            if (!wait(empty_a + xs * 8, parity)) return false;
-            const uint32_t at = xs * x_slot;
-            uint32_t n[kXB], off[kXB];   // bytes and columns; behind the last block, and behind the last column in it, zeros
+        return in_order(q, w, [&](uint32_t kb, uint32_t xs, uint32_t par) -> bool {
+          if (!wait(empty_a + xs * 8, par)) return false;
+          const uint32_t at = xs * x_slot;
+          uint32_t n[kXB], off[kXB];   // bytes and columns; behind the last block, and behind the last column in it, zeros
 #pragma unroll
-            for (uint32_t b = 0; b < kXB; ++b) {
-              const bool in = kb + b < w.kb1 && (kb + b) * 64u + c * 8u < K;
-              n[b] = in ? 16u : 0u;
-              off[b] = in ? b * 64u : 0u;
-            }
-            const __nv_bfloat16* src = x0 + (n[0] ? kb * 64u : 0u);
-#pragma unroll
-            for (uint32_t i = 0; i < kN / 8; ++i) {
-              if (i * 8 + r0 < M_b) {
-#pragma unroll
-                for (uint32_t b = 0; b < kXB; ++b) cp_async_16s(to0 + at + i * 1024u + b * x_block, src + off[b], n[b]);
-              }
-              src += (size_t)4 * K;
-              if (i * 8 + 4 + r0 < M_b) {
-#pragma unroll
-                for (uint32_t b = 0; b < kXB; ++b) cp_async_16s(to1 + at + i * 1024u + b * x_block, src + off[b], n[b]);
-              }
-              src += (size_t)4 * K;
-            }
-            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(full_a + xs * 8) : "memory");
-            if (++xs == x_slots) { xs = 0; parity ^= 1u; }
+          for (uint32_t b = 0; b < kXB; ++b) {
+            const bool in = kb + b < w.kb1 && (kb + b) * 64u + c * 8u < K;
+            n[b] = in ? 16u : 0u;
+            off[b] = in ? b * 64u : 0u;
           }
+          const __nv_bfloat16* src = x0 + (n[0] ? kb * 64u : 0u);
+#pragma unroll
+          for (uint32_t i = 0; i < kN / 8; ++i) {
+            if (i * 8 + r0 < M_b) {
+#pragma unroll
+              for (uint32_t b = 0; b < kXB; ++b) cp_async_16s(to0 + at + i * 1024u + b * x_block, src + off[b], n[b]);
+            }
+            src += (size_t)4 * K;
+            if (i * 8 + 4 + r0 < M_b) {
+#pragma unroll
+              for (uint32_t b = 0; b < kXB; ++b) cp_async_16s(to1 + at + i * 1024u + b * x_block, src + off[b], n[b]);
+            }
+            src += (size_t)4 * K;
+          }
+          asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(full_a + xs * 8) : "memory");
+          return true;
+        });
       }
-      return true;
     };
     for (uint32_t ph = 0; ph < p.n_phases; ++ph) {
       if (ph > 0) {
@@ -527,21 +572,28 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
       if (!produce(p.ph[ph], ph)) break;
     }
     if constexpr (!kTmaX) cp_async_wait_all();   // (nothing in flight when the shared memory goes away)
-  } else if (warp == 2) {
+  } else if (warp == 2 || warp == kEpiWarp0 + kEpiWarps) {
     // ------------------------------------------------------------------ MMA issue
-    // This warp's instruction latency is what bounds a product whose operands are in place (measured with
-    // the MMAs left out: 550 - 630 cycles per stage with one wait after the other and 64-bit
-    // descriptors, where HBM delivers a stage of a short product in 590): the two barriers of an
-    // iteration are polled by one instruction, and descriptors are stepped in 32 bits.
+    // A warp cannot run ahead of the tensor cores by more than an MMA or two, so everything it does between
+    // two groups of MMAs - barriers polled, commits (the second of a pair alone 73 cycles), the loop - adds
+    // to their time unless another warp's MMAs fill it: hence the second pipeline.  Cycles per k block
+    // (4 MMAs) with the operands always in place, 64 x 8 / 128 x 16 / 128 x 128 / 128 x 256 results: one warp
+    // 383 / 428 / 473 / 535, two 192 / 216 / 256 / 512; the MMAs themselves take 92 / 156 / 256 / 512, and HBM
+    // delivers the weights of one in 275 / 490 / 490 / 490.
+    // (A pipeline's barriers have one consumer.  Two warps that took the stages of one ring in turn would poll
+    // barriers whose earlier phases they have not seen, which a parity cannot tell from the one meant.)
     // (idesc64: an image of 8 alone, 64 rows)
+    const uint32_t pipe = warp == 2 ? 0u : 1u, first = pipe * pipe_stages, first_x = pipe * pipe_slots;
     const uint32_t idesc = umma_idesc_bf16_f32(kRowTile, nb < 16 ? 16 : nb);
     const uint32_t idesc64 = umma_idesc_bf16_f32(kRowTile / 2, nb);
-    const uint32_t full_a = smem_u32(w_full), empty_a = smem_u32(w_empty), xfull_a = smem_u32(x_full), xempty_a = smem_u32(x_empty);
-    const uint32_t w_low = desc_low(smem_u32(ring)), x_low = desc_low(smem_u32(x_ring)), x_step = x_slot / 16, x_half = x_block / 16;
+    const uint32_t full_a = smem_u32(w_full) + first * 8, empty_a = smem_u32(w_empty) + first * 8;
+    const uint32_t xfull_a = smem_u32(x_full) + first_x * 8, xempty_a = smem_u32(x_empty) + first_x * 8;
+    const uint32_t x_step = x_slot / 16, x_half = x_block / 16;
+    const uint32_t w_low = desc_low(smem_u32(ring) + first * kStageBytes), x_low = desc_low(smem_u32(x_ring) + first_x * x_slot);
     const uint32_t afull_a = smem_u32(acc_full), aempty_a = smem_u32(acc_empty);
     uint32_t stage = 0, parity = 0, xs = 0, xpar = 0, as = 0, apar = 1;
-    auto next_stage = [&]() { if (++stage == n_stages) { stage = 0; parity ^= 1u; } };
-    auto next_slot = [&]() { if (++xs == x_slots) { xs = 0; xpar ^= 1u; } };
+    auto next_stage = [&]() { if (++stage == pipe_stages) { stage = 0; parity ^= 1u; } };
+    auto next_slot = [&]() { if (++xs == pipe_slots) { xs = 0; xpar ^= 1u; } };
     auto next_acc = [&]() { if (++as == kSlots) { as = 0; apar ^= 1u; } };
     // odd lanes poll one barrier, even lanes the other
     auto wait_two = [&](uint32_t bar0, uint32_t par0, uint32_t bar1, uint32_t par1) -> bool {
@@ -552,17 +604,16 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
       return __all_sync(0xFFFFFFFFu, ok) != 0;
     };
     auto wait_one = [&](uint32_t bar, uint32_t par) -> bool { return wait_two(bar, par, bar, par); };
-    auto wait_three = [&](uint32_t bar0, uint32_t par0, uint32_t bar1, uint32_t par1, uint32_t bar2, uint32_t par2) -> bool {
-      return wait_two(bar0, par0, (lane & 2u) ? bar2 : bar1, (lane & 2u) ? par2 : par1);
-    };
-    // image8: images of 8 units (two k blocks a stage).  mode: parts of a quarter of a k block (0), a k block (1), several (2).
-    // (Compile-time, and slots around the loop over stages, for this warp's instruction latency: with one
-    // loop that decides at run time a step of one sequence took 4230 us instead of 3570, all else equal.)
+    // image8: images of 8 units (two k blocks a stage).  mode: see PairPhase.  (Compile-time, for this
+    // warp's instruction latency.)
     auto multiply = [&](const PairPhase& q, auto image8, auto mode) -> bool {
       constexpr bool kImage8 = decltype(image8)::value;
       constexpr uint32_t kMode = decltype(mode)::value;
+      // k blocks of an iteration (one pipeline: of an image of 8 in slots of one block, half a stage)
+      constexpr uint32_t kStep = kPipes == 1 ? (kImage8 && kMode == 2 ? 2 : 1) : chunk_blocks(kN, kImage8 ? 8 : 16);
+      constexpr bool kHalves = kImage8 && kStep == 1;
       const Part w = part_of(q);
-      const uint32_t slot_n = slot_blocks(kN, kMode == 2 ? q.part_blocks : kMode), id = kImage8 ? idesc64 : idesc;
+      const uint32_t slot_n = q.slot_blocks, id = kImage8 ? idesc64 : idesc;
       constexpr uint32_t kBlockCols = kMode == 2 ? 0 : kMode == 1 ? part_cols(kN) : 4 * part_cols(kN), kNext = kMode == 0 ? part_cols(kN) : 0;
       // One k block: 4 MMAs.  (16 columns on: 32 bytes, 2 in a descriptor's address field, which counts in 16 bytes)
       auto mma_block = [&](uint32_t d, uint32_t wl, uint32_t xl, uint32_t accumulate) {
@@ -571,135 +622,52 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
           umma_low(d + ks * kNext, wl + 2 * ks, xl + 2 * ks, id, kMode == 0 ? 0u : ks == 0 ? accumulate : 1u);
       };
       for (uint32_t ua = w.u0; ua < w.u1; ua += w.run) {
-        for (uint32_t kb = w.kb0; kb < w.kb1;) {   // a slot of accumulators: the epilogue warps have read what was there
-          const uint32_t kb_end = min(kb + slot_n, w.kb1), done = afull_a + as * 8;
-          [[maybe_unused]] const uint32_t kb_first = kb;
-          uint32_t d = tmem + as * kSlotCols, accumulate = 0;
-          if constexpr (kMode != 0)
-            if (!wait_one(aempty_a + as * 8, apar)) return false;
-          if constexpr (kXB == 4) {
-            constexpr uint32_t kPer = kImage8 ? 2 : 1;   // k blocks of a stage
-            for (; kb < kb_end; kb += kXB) {
-              const uint32_t n = min(kXB, kb_end - kb), xl = x_low + xs * x_step, free_x = xempty_a + xs * 8;
-#pragma unroll
-              for (uint32_t j = 0; j < kXB; j += kPer) {
-                if (j && j >= n) break;
-                const uint32_t wl = w_low + stage * (kStageBytes / 16), full_w = full_a + stage * 8, free_w = empty_a + stage * 8;
-                const bool last = j + kPer >= n;
-                bool ok;
-                if (j) ok = wait_one(full_w, parity);
-                else if (kMode == 0 && kb == kb_first) ok = wait_three(full_w, parity, xfull_a + xs * 8, xpar, aempty_a + as * 8, apar);
-                else ok = wait_two(full_w, parity, xfull_a + xs * 8, xpar);
-                if (!ok) return false;
-                if (j == 0) fence_proxy_async_smem();   // (activations that came through the load/store path)
-                tc_fence_after_sync();
-                next_stage();
-                if (elect_one()) {
-                  mma_block(d + j * kBlockCols, wl, xl + j * x_half, j ? kMode == 2 : accumulate);
-                  if (kImage8 && j + 1 < n) mma_block(d + (j + 1) * kBlockCols, wl + kStageBytes / 32, xl + (j + 1) * x_half, kMode == 2);
-                  commit(free_w);
-                  if (last) commit(free_x);
-                  if (kMode == 0 && last && kb + kXB >= kb_end) commit(done);
-                }
-                __syncwarp();
-              }
-              next_slot();
-              d += kXB * kBlockCols;
-              accumulate = kMode == 2;
-            }
-            kb = kb_end;
-          } else if constexpr (kXB == 2) {
-            for (; kb < kb_end; kb += 2) {
-              const uint32_t wl = w_low + stage * (kStageBytes / 16), xl = x_low + xs * x_step;
-              const uint32_t free0 = empty_a + stage * 8, free_x = xempty_a + xs * 8;
-              if (!wait_two(full_a + stage * 8, parity, xfull_a + xs * 8, xpar)) return false;
-              if constexpr (!kTmaX) fence_proxy_async_smem();
-              tc_fence_after_sync();
-              next_stage();
-              next_slot();
-              if constexpr (kImage8) {
-                if (elect_one()) {
-                  mma_block(d, wl, xl, accumulate);
-                  if (kb + 1 < w.kb1) mma_block(d + kBlockCols, wl + kStageBytes / 32, xl + x_half, kMode == 2);
-                  commit(free0);
-                  commit(free_x);
-                }
-              } else {
-                const bool both = kb + 1 < w.kb1;
-                if (elect_one()) {
-                  mma_block(d, wl, xl, accumulate);
-                  commit(free0);
-                  if (!both) commit(free_x);
-                }
-                __syncwarp();
-                if (both) {
-                  const uint32_t wl1 = w_low + stage * (kStageBytes / 16), free1 = empty_a + stage * 8;
-                  if (!wait_one(full_a + stage * 8, parity)) return false;
-                  tc_fence_after_sync();
-                  next_stage();
-                  if (elect_one()) {
-                    mma_block(d + kBlockCols, wl1, xl + x_half, kMode == 2);
-                    commit(free1);
-                    commit(free_x);
-                  }
-                }
-              }
-              __syncwarp();
-              d += 2 * kBlockCols;
-              accumulate = kMode == 2;
-            }
-          } else if constexpr (kImage8 && kMode == 2) {
-            for (; kb < kb_end; kb += 2) {   // (the activation tiles of a stage's two k blocks are slots of their own)
-              const bool both = kb + 1 < w.kb1;
-              const uint32_t wl = w_low + stage * (kStageBytes / 16), xl = x_low + xs * x_step;
-              const uint32_t free_w = empty_a + stage * 8, free_x = xempty_a + xs * 8;
-              if (!wait_two(full_a + stage * 8, parity, xfull_a + xs * 8, xpar)) return false;
-              tc_fence_after_sync();
-              next_stage();
-              next_slot();
+        for (uint32_t k0 = w.kb0; k0 < w.kb1; k0 += slot_n) {   // a slot of accumulators: the epilogue warps have read what was there
+          const uint32_t k1 = min(k0 + slot_n, w.kb1), done = afull_a + as * 8;
+          uint32_t d = tmem + as * kSlotCols + pipe * (kMode == 2 ? part_cols(kN) : kStep * kBlockCols), accumulate = 0;
+          if (!wait_one(aempty_a + as * 8, apar)) return false;
+          for (uint32_t kb = k0 + pipe * kStep; kb < k1; kb += kPipes * kStep, d += kPipes * kStep * kBlockCols) {
+            const bool both = kStep == 2 && kb + 1 < k1, second = kHalves && ((kb - w.kb0) & 1u), last = !kHalves || second || kb + 1 == w.kb1;
+            const uint32_t wl = w_low + stage * (kStageBytes / 16) + (second ? kStageBytes / 32 : 0u), xl = x_low + xs * x_step;
+            const uint32_t free_w = empty_a + stage * 8, free_x = xempty_a + xs * 8;
+            if (!wait_two(full_a + stage * 8, parity, xfull_a + xs * 8, xpar)) return false;
+            if constexpr (!kTmaX) fence_proxy_async_smem();   // (activations that came through the load/store path)
+            tc_fence_after_sync();
+            if (last) next_stage();
+            next_slot();
+            if constexpr (kStep == 1 || (kImage8 && kXB == 2)) {   // one stage, one activation slot
               if (elect_one()) {
                 mma_block(d, wl, xl, accumulate);
+                if (both) mma_block(d + kBlockCols, wl + kStageBytes / 32, xl + x_half, kMode == 2);
+                if (last) commit(free_w);
                 commit(free_x);
-                if (!both) commit(free_w);
+              }
+              __syncwarp();
+            } else {   // two stages of one k block, or (from 128 rows on) two activation slots of one
+              if (elect_one()) {
+                mma_block(d, wl, xl, accumulate);
+                if (!kImage8 || !both) commit(free_w);
+                if (kXB == 1 || !both) commit(free_x);
               }
               __syncwarp();
               if (both) {
-                const uint32_t xl1 = x_low + xs * x_step, free_x1 = xempty_a + xs * 8;
-                if (!wait_one(xfull_a + xs * 8, xpar)) return false;
+                const uint32_t wl1 = kImage8 ? wl + kStageBytes / 32 : w_low + stage * (kStageBytes / 16), free_w1 = kImage8 ? free_w : empty_a + stage * 8;
+                const uint32_t xl1 = kXB == 2 ? xl + x_half : x_low + xs * x_step, free_x1 = kXB == 2 ? free_x : xempty_a + xs * 8;
+                if (!(kImage8 ? wait_one(xfull_a + xs * 8, xpar) : wait_one(full_a + stage * 8, parity))) return false;
                 tc_fence_after_sync();
-                next_slot();
+                if constexpr (kImage8) next_slot(); else next_stage();
                 if (elect_one()) {
-                  mma_block(d, wl + kStageBytes / 32, xl1, 1u);
+                  mma_block(d + kBlockCols, wl1, xl1, kMode == 2);
+                  commit(free_w1);
                   commit(free_x1);
-                  commit(free_w);
                 }
                 __syncwarp();
               }
-              accumulate = 1;
             }
-          } else {
-            for (; kb < kb_end; ++kb) {   // (a part is a k block: an image of 8 may leave a slot in the middle of a stage)
-              const bool second = kImage8 && ((kb - w.kb0) & 1u), last = !kImage8 || second || kb + 1 == w.kb1;
-              const uint32_t wl = w_low + stage * (kStageBytes / 16) + (second ? kStageBytes / 32 : 0u), xl = x_low + xs * x_step;
-              const uint32_t free_w = empty_a + stage * 8, free_x = xempty_a + xs * 8;
-              if (!wait_two(full_a + stage * 8, parity, xfull_a + xs * 8, xpar)) return false;
-              tc_fence_after_sync();
-              if (last) next_stage();
-              next_slot();
-              if (elect_one()) {
-                mma_block(d, wl, xl, accumulate);
-                commit(free_x);
-                if (last) commit(free_w);
-              }
-              __syncwarp();
-              d += kBlockCols;
-              accumulate = kMode == 2;
-            }
+            accumulate = kMode == 2;
           }
-          if constexpr (kMode != 0) {
-            if (elect_one()) commit(done);
-            __syncwarp();
-          }
+          if (elect_one()) commit(done);   // (a warp that had no chunk arrives all the same)
+          __syncwarp();
           next_acc();
         }
       }
@@ -708,8 +676,8 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
     auto multiply_phase = [&](const PairPhase& q) -> bool {
       auto with_mode = [&](auto mode) { return q.image == 8 ? multiply(q, Const<true>(), mode) : multiply(q, Const<false>(), mode); };
       if constexpr (kN == 8)
-        if (q.part_blocks == 0) return with_mode(Const<0u>());
-      return q.part_blocks == 1 ? with_mode(Const<1u>()) : with_mode(Const<2u>());
+        if (q.mode == 0) return with_mode(Const<0u>());
+      return q.mode == 1 ? with_mode(Const<1u>()) : with_mode(Const<2u>());
     };
     for (uint32_t ph = 0; ph < p.n_phases; ++ph)
       if (!multiply_phase(p.ph[ph])) break;
@@ -917,37 +885,29 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
       constexpr uint32_t kGroups = kN / (HG * CH);
       auto column = [&](uint32_t i) { return hh * CH + i * (HG * CH); };
       const uint32_t lane_base = tmem + ((quarter * 32u) << 16);
-      const uint32_t part_blocks = q.part_blocks, slot_n = slot_blocks(kN, part_blocks);
+      const uint32_t mode = q.mode, slot_n = q.slot_blocks;
+      // Parts of a slot with this many k blocks.
+      auto parts_of = [&](uint32_t blocks) -> uint32_t {
+        if (mode != 2) return mode ? blocks : 4 * blocks;
+        return kPipes == 2 && blocks > chunk_blocks(kN, image) ? 2u : 1u;
+      };
+      auto wait_slot = [&]() {
+        wait(smem_u32(&acc_full[as]), apar);
+        __syncwarp();
+        tc_fence_after_sync();
+      };
+      auto next_slot = [&]() { if (++as == kSlots) { as = 0; apar ^= 1u; } };
       // From 128 rows on the sums would be up to half of a thread's registers: they stay in tensor memory, in
       // the slot of the last part added, which is given back when the epilogue has read them.  (Registers:
       // 244 - 508 bytes of spills at 256 rows, 6-layer step at batch 250 2147 - 2350 us instead of 2045.)
       constexpr bool kParkSums = kN >= 128;
       float sum[kParkSums ? 1 : kGroups][CH];
       uint32_t parked = 0;   // the slot kept
+      [[maybe_unused]] bool parked_two = false;   // it holds two parts, whose sum is still to be taken
       auto release_slot = [&](uint32_t slot) {
         tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(&acc_empty[slot]);
-      };
-      auto group_sums = [&](uint32_t i, float (&v)[CH]) {   // i: a constant, except where the sums are parked
-        if constexpr (kParkSums) {
-          tmem_ld_8(lane_base + parked * kSlotCols + column(i), v);
-        } else {
-#pragma unroll
-          for (uint32_t e = 0; e < CH; ++e) v[e] = sum[i][e];
-        }
-      };
-      // Every part of the image's columns, as its slot comes.  take(from, n): the n parts at tensor-memory address `from`.
-      auto each_slot = [&](auto take) {
-        for (uint32_t kb = w.kb0; kb < w.kb1; kb += slot_n) {
-          wait(smem_u32(&acc_full[as]), apar);
-          __syncwarp();
-          tc_fence_after_sync();
-          const uint32_t here = min(slot_n, w.kb1 - kb);
-          if (column(0) < M_b) take(lane_base + as * kSlotCols + column(0), part_blocks > 1 ? 1u : part_blocks ? here : 4 * here);
-          release_slot(as);
-          if (++as == kSlots) { as = 0; apar ^= 1u; }
-        }
       };
       auto add = [&](float* to, const float* v, uint32_t n) {
 #pragma unroll
@@ -957,13 +917,38 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
           to[j + 1] = t.y;
         }
       };
+      auto group_sums = [&](uint32_t i, float (&v)[CH]) {   // i: a constant, except where the sums are parked
+        if constexpr (kParkSums) {
+          const uint32_t at = lane_base + parked * kSlotCols + column(i);
+          if (kPipes == 2 && parked_two) {
+            float both[16];
+            tmem_ld_2x8(at, at + part_cols(kN), both);
+            add(both, both + 8, 8);
+#pragma unroll
+            for (uint32_t e = 0; e < 8; ++e) v[e] = both[e];
+          } else {
+            tmem_ld_8(at, v);
+          }
+        } else {
+#pragma unroll
+          for (uint32_t e = 0; e < CH; ++e) v[e] = sum[i][e];
+        }
+      };
+      // Every part of the image's columns, as its slot comes.  take(from, n): the n parts at tensor-memory address `from`.
+      auto each_slot = [&](auto take) {
+        for (uint32_t kb = w.kb0; kb < w.kb1; kb += slot_n) {
+          wait_slot();
+          if (column(0) < M_b) take(lane_base + as * kSlotCols + column(0), parts_of(min(slot_n, w.kb1 - kb)));
+          release_slot(as);
+          next_slot();
+        }
+      };
       auto accumulate = [&]() {
         if constexpr (kParkSums) {
-          for (uint32_t kb = w.kb0; kb < w.kb1; kb += slot_n) {   // (a slot is one part)
-            wait(smem_u32(&acc_full[as]), apar);
-            __syncwarp();
-            tc_fence_after_sync();
-            if (kb != w.kb0) {   // the sum so far, from the slot before, goes on top of this part
+          for (uint32_t kb = w.kb0; kb < w.kb1; kb += slot_n) {   // (one or two parts a slot)
+            wait_slot();
+            const bool two_parts = parts_of(min(slot_n, w.kb1 - kb)) == 2;
+            if (kb != w.kb0) {   // the sum so far, from the slot before, goes on top of this slot's first part
               const uint32_t before = lane_base + parked * kSlotCols, here = lane_base + as * kSlotCols;
 #pragma unroll
               for (uint32_t i = 0; i < kGroups; ++i) {
@@ -971,13 +956,24 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
                 float v[16];
                 tmem_ld_2x8(before + column(i), here + column(i), v);
                 add(v, v + 8, 8);
+                if constexpr (kPipes == 2) {
+                  if (parked_two) {
+                    tmem_ld_8(before + part_cols(kN) + column(i), reinterpret_cast<float(&)[8]>(v[8]));
+                    add(v, v + 8, 8);
+                  }
+                  if (two_parts) {
+                    tmem_ld_8(here + part_cols(kN) + column(i), reinterpret_cast<float(&)[8]>(v[8]));
+                    add(v, v + 8, 8);
+                  }
+                }
                 tmem_st_8(here + column(i), v);
               }
               tmem_st_wait();
               release_slot(parked);
             }
             parked = as;
-            if (++as == kSlots) { as = 0; apar ^= 1u; }
+            parked_two = two_parts && kb == w.kb0;
+            next_slot();
           }
         } else {
 #pragma unroll
@@ -985,7 +981,7 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
 #pragma unroll
             for (uint32_t j = 0; j < CH; ++j) sum[i][j] = 0.f;
           if constexpr (kN == 8) {
-            if (part_blocks == 0) {
+            if (mode == 0) {
               // batches of 1 and 2, whose sums compare with those of CUDA cores: four parts added up pairwise,
               // then a compensated sum (Knuth's two-sum: t + error = s + p exactly)
               float2 s = make_float2(0.f, 0.f), lost = s;
@@ -1171,18 +1167,25 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
     // may be in the tensor cores' pipeline or on its way to shared memory when that goes away.  Each
     // issuer waits, as long as any other wait, for what it has started.  (A fixed time would not do: over
     // the host link the copies in flight of all threadblocks are a third of a millisecond.)
-    if (warp == 2) {
-      if (elect_one()) commit(smem_u32(&drained));
+    if (warp == 2 || warp == kEpiWarp0 + kEpiWarps) {
+      uint64_t* const bar = &drained[warp == 2 ? 0 : 1];
+      if (elect_one()) commit(smem_u32(bar));
       __syncwarp();
-      mbar_wait(&drained, 0, status);
+      mbar_wait(bar, 0, status);
     } else if (warp < kEpiWarp0 && (warp != 1 || kTmaX)) {
       // the last use of every stage, backwards from the next one (uses before the first count as landed)
-      const uint32_t n = warp == 1 ? x_slots : n_stages;
+      const uint32_t n = warp == 1 ? pipe_slots : pipe_stages;
+      uint64_t* const full = warp == 1 ? x_full : w_full + (kPipes == 2 && warp == 3 ? pipe_stages : 0);
       for (uint32_t i = 0; i < n; ++i) {
         if (stage == 0) { stage = n; parity ^= 1u; }
         --stage;
-        if (warp != 1) my_turn = !my_turn;
-        if (my_turn) mbar_wait(warp == 1 ? &x_full[stage] : &w_full[stage], parity ^ 1u, status);
+        if (kPipes == 1 && warp != 1) my_turn = !my_turn;
+        if (my_turn) mbar_wait(full + stage, parity ^ 1u, status);
+        if (kPipes == 2 && warp == 1) {
+          if (stage1 == 0) { stage1 = n; parity1 ^= 1u; }
+          --stage1;
+          mbar_wait(full + n + stage1, parity1 ^ 1u, status);
+        }
       }
     }
     __syncthreads();
@@ -1195,38 +1198,41 @@ __global__ void __maxnreg__(96) gemv_pair_kernel(const __grid_constant__ PairPar
 uint32_t units_bound(uint32_t n_units, uint32_t W) { return (n_units + W - 1) / W; }
 uint32_t images_bound(uint32_t n_units, uint32_t W) { return (units_bound(n_units, W) + 15) / 16; }
 
-// k blocks of an accumulator.  Every hand-over costs the MMA warp 350 cycles and more (output product
-// at batch 32: 2800 of 14000 with eight), so parts are as long as the results allow:
+// The k blocks of an accumulator, and with them the slots.  Every hand-over costs the MMA warps 350
+// cycles and more, so accumulators hold as many as the results allow:
 //   fp32 results   0.9 of the threadblocks' segments in the kernels of kernels_gemv.cu (two per SM up
 //                  to 128 rows, one above; none longer than a row tile's columns): the sums are then no
 //                  further from the exact ones than theirs.  Batches of 1 and 2, whose segments are
 //                  summed on CUDA cores there: a quarter of a block.
 //   bf16 results   at least 4096 columns (as many as those segments have at most): 4.4e-6 of the sum,
 //                  where the rounding behind it is 1.7e-3.
-// An even number (up to 16 rows a multiple of four: whole activation slots), or 1.
-uint32_t part_blocks_of(const PairPhase& q, uint32_t clusters, uint32_t M_b) {
+// An even number (up to 16 rows a multiple of four), or 1.  A slot has an accumulator per pipeline.
+void plan_parts(PairPhase& q, uint32_t clusters, uint32_t n_class, uint32_t M_b) {
   const bool fp32 = q.epi == BOOST_EPI_PLAIN && q.y_dtype == 0;
-  if (fp32 && M_b <= 2) return 0;
+  q.mode = fp32 && M_b <= 2 ? 0 : 1;
+  q.slot_blocks = q.mode == 0 ? slot_parts(n_class) / 4 : slot_parts(n_class);
   const uint64_t blocks = (uint64_t)(q.n_units / kUnitsPerTile) * q.k_blocks, segments = (uint64_t)clusters * (M_b <= 128 ? 4 : 2);
   uint32_t n = (uint32_t)(9 * (blocks < segments * q.k_blocks ? blocks : segments * q.k_blocks) / (10 * segments));
   if (!fp32 && n < 64) n = 64;
   const uint32_t unit = M_b <= 16 ? 4 : 2;
-  n = n / unit * unit;
-  if (n == 0) return 1;
-  const uint32_t own = (q.k_blocks + q.split - 1) / q.split, parts = (own + n - 1) / n;   // parts as even as they come
-  return ((own + parts - 1) / parts + unit - 1) / unit * unit;
+  n = n / unit * unit * pipes_of(n_class);
+  if (q.mode == 0 || n == 0) return;
+  q.mode = 2;
+  const uint32_t own = (q.k_blocks + q.split - 1) / q.split, slots = (own + n - 1) / n;   // slots as even as they come
+  const uint32_t round = pipes_of(n_class) == 2 ? 2 * chunk_blocks(n_class, q.image) : 2;
+  q.slot_blocks = ((own + slots - 1) / slots + round - 1) / round * round;
 }
 
 // How a phase is cut.  Two threadblocks share the rows of a cluster, half of K each, where those rows
 // fit one image: little crosses between them, and the rows divide evenly (4096 rows over 74
 // clusters: 98.8 % of the SMs' time, over 148 threadblocks 86 %).  Longer products (gate / up, LM head)
 // have rows enough for every threadblock on its own (97 % and more) and nothing to exchange.
-void plan_phase(PairPhase& q, uint32_t clusters, uint32_t M_b) {
+void plan_phase(PairPhase& q, uint32_t clusters, uint32_t n_class, uint32_t M_b) {
   q.split = (q.k_blocks >= 2 && units_bound(q.n_units, clusters) <= 16) ? 2u : 1u;
   const uint32_t W = q.split == 2 ? clusters : 2 * clusters;
   q.image = units_bound(q.n_units, W) <= 8 ? 8u : 16u;
   q.max_images = images_bound(q.n_units, W);
-  q.part_blocks = part_blocks_of(q, clusters, M_b);
+  plan_parts(q, clusters, n_class, M_b);
 }
 uint32_t ssq_parts_of(const PairPhase& q, uint32_t clusters) { return (q.split == 2 ? clusters : 2 * clusters) * q.max_images * (q.image / 8); }
 
@@ -1296,18 +1302,20 @@ int launch_pair(PairParams& p, float* stats, size_t stats_bytes, cudaStream_t st
   // activation slots: more than a microsecond of a short product's stream (a k block per 155 ns); from
   // 128 rows on about half of the shared memory, since the tiles are as large as the weight stages
   const uint32_t slot_bytes = x_blocks(kN) * p.nb * 128u;
-  const uint32_t x_budget = kN <= 16 ? 3 * slot_bytes : kN == 32 ? 4 * slot_bytes : kN == 64 ? 64u * 1024u : 96u * 1024u;
+  const uint32_t x_budget = kN <= 16 ? 6 * slot_bytes : kN == 32 ? 4 * slot_bytes : kN == 64 ? 64u * 1024u : 96u * 1024u;
   p.x_slots = x_budget / slot_bytes < kMaxXSlots ? x_budget / slot_bytes : kMaxXSlots;
+  p.x_slots = p.x_slots / pipes_of(kN) * pipes_of(kN);
   const uint32_t fixed = 2048u + p.x_slots * slot_bytes + sums_bytes(kN);
   p.n_stages = (smem_total(kN) - fixed) / kStageBytes;
   if (p.n_stages > kMaxStages) p.n_stages = kMaxStages;
+  p.n_stages = p.n_stages / pipes_of(kN) * pipes_of(kN);
   const size_t smem = smem_total(kN);
   // (the caller's ssq pointers stand in for the buffers until here)
   const float* key[kMaxPhases];
   uint32_t n_stats = 0;
   for (uint32_t i = 0; i < p.n_phases; ++i) {
     PairPhase& q = p.ph[i];
-    plan_phase(q, clusters, p.M_b);
+    plan_phase(q, clusters, kN, p.M_b);
     for (int j = (int)i - 1; j >= 0; --j)
       if (q.ssq_in && key[j] == q.ssq_in) {
         q.ssq_in = p.ph[j].ssq_out;
@@ -1344,7 +1352,7 @@ boosth::PairCut boosth::pair_cut(uint32_t N, uint32_t K, uint32_t M_b) {
   q.k_blocks = (K + 63) / 64;
   q.n_units = (N + kRowTile - 1) / kRowTile * kUnitsPerTile;
   const uint32_t clusters = clusters_for(M_b);
-  plan_phase(q, clusters, M_b);
+  plan_phase(q, clusters, batch_class(M_b), M_b);
   return {2 * clusters, q.split, units_bound(q.n_units, q.split == 2 ? clusters : 2 * clusters)};
 }
 
