@@ -32,8 +32,8 @@
 //
 // Warps: 0 and 3 weight producers (a pipeline each, or every other stage: one warp's instruction latency
 // would bound the stream of a product whose stages are four or eight copies), 1 activation producer, 2 MMA
-// issue and tensor-memory allocation, 4 and up epilogue, the last one (up to 128 rows) the second pipeline's
-// MMA issue.  Producers and MMA warps run warp-uniform code and elect a lane for the copy or MMA itself: inside an if (lane == 0) every operand goes through a
+// issue and tensor-memory allocation, 4 and up epilogue, behind them (up to 128 rows) the second
+// pipeline's MMA issue and (128 rows) activation producer.  Producers and MMA warps run warp-uniform code and elect a lane for the copy or MMA itself: inside an if (lane == 0) every operand goes through a
 // vector register (measured: a group of four MMAs and a commit 293 cycles against 212, a bulk copy 64
 // against 25).
 #include <cuda.h>
@@ -121,10 +121,13 @@ __host__ __device__ constexpr uint32_t tmem_cols(uint32_t n) { return acc_slots(
 __host__ __device__ constexpr uint32_t chunk_blocks(uint32_t n, uint32_t image) {
   return pipes_of(n) == 1 ? 1 : image == 8 || x_blocks(n) == 2 ? 2 : 1;
 }
+// Activation producers.  (At 128 rows one is too slow for both pipelines: 375 cycles a slot, where the tensor cores take
+// 256 and HBM 275; down product 34.2 -> 30.2 us with two.  Fewer rows: slots of two blocks; batch 64 was 0.6 % slower with two.)
+__host__ __device__ constexpr uint32_t x_warps(uint32_t n) { return n == 128 ? 2 : 1; }
 // Epilogue warps: a short product's last accumulator is finished by all of them at the end of a phase,
 // which at large batches is bound by their instruction latency.
 __host__ __device__ constexpr uint32_t epi_warps(uint32_t n) { return n <= 32 ? 8 : 16; }
-__host__ __device__ constexpr uint32_t threads_of(uint32_t n) { return (kEpiWarp0 + epi_warps(n) + pipes_of(n) - 1) * 32; }
+__host__ __device__ constexpr uint32_t threads_of(uint32_t n) { return (kEpiWarp0 + epi_warps(n) + pipes_of(n) - 1 + x_warps(n) - 1) * 32; }
 // Sums on their way from tensor memory to the threads that finish them, fp32 [columns][128 lanes].
 // Rows of one threadblock: this many columns at a time (32 in two buffers in turn were 1.5 % slower than 64
 // for a step at batch 250).  128 rows: 32, so that shared memory holds six stages and six activation slots
@@ -132,7 +135,8 @@ __host__ __device__ constexpr uint32_t threads_of(uint32_t n) { return (kEpiWarp
 __host__ __device__ constexpr uint32_t chunk_cols(uint32_t n) { return n < 64 ? n : n == 128 ? 32 : 64; }
 // Rows that two threadblocks share: each finishes half of the columns, in this many rounds.  The
 // columns of a round, this threadblock's sums and the peer's, are kept in the chunk buffers
-// (up to 32 rows) or in the activation slots, which are idle then.
+// (up to 32 rows), or this threadblock's in the activation slots, which are idle then, and the peer's in the
+// chunk buffer where they fit (64 and 128 rows).
 __host__ __device__ constexpr uint32_t rounds_of(uint32_t n) { return n >= 256 ? 2 : 1; }
 __host__ __device__ constexpr uint32_t sums_bytes(uint32_t n) { return chunk_cols(n) * kRowTile * 4; }
 
@@ -374,9 +378,10 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
   };
   // A pipeline's stages (activation slots) are behind each other.
   const uint32_t pipe_stages = n_stages / kPipes, pipe_slots = x_slots / kPipes;
+  constexpr uint32_t kMma1 = kEpiWarp0 + kEpiWarps, kX1 = kMma1 + 1;   // the second pipeline's MMA warp and activation producer
   // Where a producer warp stands: the stage (activation slot) it would fill next, the parity of its wait for
-  // it (the activation producer's second pipeline: stage1, parity1), and whether it is this warp's turn.
-  // Known at the end of the kernel too, for the wind-down.
+  // it (one activation producer for two pipelines: stage1, parity1 for the second), and whether it is this
+  // warp's turn.  Known at the end of the kernel too, for the wind-down.
   uint32_t stage = 0, parity = 1;
   [[maybe_unused]] uint32_t stage1 = 0, parity1 = 1;
   bool my_turn = kPipes == 2 || warp != 3;
@@ -464,11 +469,12 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
     };
     for (uint32_t ph = 0; ph < p.n_phases; ++ph)
       if (!produce(p.ph[ph], ph)) break;
-  } else if (warp == 1) {
-    // ------------------------------------------------------------------ activation producer
+  } else if (warp == 1 || warp == kX1) {
+    // ------------------------------------------------------------------ activation producers
     // Up to 32 rows: 16-byte copies through the load/store path (the TMA unit works in order, and an
     // activation tile would queue behind the weight copies of a full ring).  Rows beyond the batch are
     // left as they are: they only reach accumulator columns that nobody reads.
+    const uint32_t pipe = warp == 1 ? 0u : 1u;
     const uint32_t x_a = smem_u32(x_ring), full_a = smem_u32(x_full), empty_a = smem_u32(x_empty);
     if constexpr (kTmaX) {
       if (elect_one())
@@ -476,27 +482,26 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
       __syncwarp();
     }
     pdl_wait();
-    // fill(kb, slot, parity): the k blocks of a slot from kb on.  For every slot of a phase, the pipelines' chunks in turn.
-    auto in_order = [&](const PairPhase& q, const Part& w, auto fill) -> bool {
-      [[maybe_unused]] const uint32_t slot_n = q.slot_blocks, chunk = chunk_blocks(kN, q.image);
+    // fill(kb, xs): the k blocks of slot xs, from kb on.  For every slot of a phase that this warp fills.
+    auto each_slot = [&](const PairPhase& q, const Part& w, auto fill) -> bool {
+      auto put = [&](uint32_t kb, uint32_t kb_end, uint32_t first, uint32_t& at, uint32_t& par) -> bool {   // into the next slots of a pipeline
+        for (; kb < kb_end; kb += kXB) {
+          if (!wait(empty_a + (first + at) * 8, par)) return false;
+          fill(kb, first + at);
+          if (++at == pipe_slots) { at = 0; par ^= 1u; }
+        }
+        return true;
+      };
       for (uint32_t pa = w.u0; pa < w.u1; pa += w.run) {
         if constexpr (kPipes == 1) {
-          for (uint32_t kb = w.kb0; kb < w.kb1; kb += kXB) {
-            if (!fill(kb, stage, parity)) return false;
-            if (++stage == pipe_slots) { stage = 0; parity ^= 1u; }
-          }
+          if (!put(w.kb0, w.kb1, 0, stage, parity)) return false;
         } else {
+          const uint32_t chunk = chunk_blocks(kN, q.image), slot_n = q.slot_blocks;
           for (uint32_t k0 = w.kb0; k0 < w.kb1; k0 += slot_n) {
             const uint32_t k1 = min(k0 + slot_n, w.kb1);
-            for (uint32_t c = k0; c < k1; c += 2 * chunk) {
-              for (uint32_t kb = c; kb < min(c + chunk, k1); kb += kXB) {
-                if (!fill(kb, stage, parity)) return false;
-                if (++stage == pipe_slots) { stage = 0; parity ^= 1u; }
-              }
-              for (uint32_t kb = c + chunk; kb < min(c + 2 * chunk, k1); kb += kXB) {
-                if (!fill(kb, pipe_slots + stage1, parity1)) return false;
-                if (++stage1 == pipe_slots) { stage1 = 0; parity1 ^= 1u; }
-              }
+            for (uint32_t c = k0 + pipe * chunk; c < k1; c += 2 * chunk) {
+              if (!put(c, min(c + chunk, k1), pipe * pipe_slots, stage, parity)) return false;
+              if (x_warps(kN) == 1 && !put(c + chunk, min(c + 2 * chunk, k1), pipe_slots, stage1, parity1)) return false;
             }
           }
         }
@@ -508,8 +513,7 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
       const uint32_t K = q.K;
       if constexpr (kTmaX) {
         fence_proxy_async_all();   // x was written with ordinary stores and is read through the TMA unit
-        return in_order(q, w, [&](uint32_t kb, uint32_t xs, uint32_t par) -> bool {
-          if (!wait(empty_a + xs * 8, par)) return false;
+        return each_slot(q, w, [&](uint32_t kb, uint32_t xs) {
           if (elect_one()) {
             const uint32_t full = full_a + xs * 8, dst = x_a + xs * x_slot;
             expect_tx(full, x_slot);
@@ -518,14 +522,12 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
             if constexpr (kXB == 2) tma_tile(dst + x_block, &p.x_map[ph], (int32_t)((kb + 1 < w.kb1 ? kb + 1 : q.k_blocks) * 64u), full);
           }
           __syncwarp();
-          return true;
         });
       } else {
         const uint32_t c = lane & 7, r0 = lane >> 3, M_b = p.M_b;
         const uint32_t to0 = x_a + r0 * 128u + ((c ^ r0) << 4), to1 = x_a + (r0 + 4) * 128u + ((c ^ (r0 + 4)) << 4);   // rows 8 i + r0, 8 i + 4 + r0
         const __nv_bfloat16* const x0 = q.x + (size_t)r0 * K + (c * 8u < K ? c * 8u : 0u);
-        return in_order(q, w, [&](uint32_t kb, uint32_t xs, uint32_t par) -> bool {
-          if (!wait(empty_a + xs * 8, par)) return false;
+        return each_slot(q, w, [&](uint32_t kb, uint32_t xs) {
           const uint32_t at = xs * x_slot;
           uint32_t n[kXB], off[kXB];   // bytes and columns; behind the last block, and behind the last column in it, zeros
 #pragma unroll
@@ -549,16 +551,16 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
             src += (size_t)4 * K;
           }
           asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(full_a + xs * 8) : "memory");
-          return true;
         });
       }
     };
     for (uint32_t ph = 0; ph < p.n_phases; ++ph) {
       if (ph > 0) {
         // one lane polls; the barrier orders the other lanes' reads behind what it has acquired
-        if (lane == 0) {
+        if (pipe) wait(smem_u32(&go), (ph - 1) & 1u);
+        else if (lane == 0) {
           if (!s_abort && !grid_counter_wait(p.bar + 1, ph * n_cta, status)) s_abort = 1;
-          mbar_arrive(&go);   // the epilogue warps may read what the phase before wrote
+          mbar_arrive(&go);   // the epilogue warps (and the second producer) may read what the phase before wrote
           // The last threadblock past the last of these waits - everybody has arrived, nobody reads the
           // counters any more - puts them back to zero for the next launch.  (Here and not at the end of
           // the kernel, where the round trip would hold up the kernel that waits for this one.)
@@ -572,7 +574,7 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
       if (!produce(p.ph[ph], ph)) break;
     }
     if constexpr (!kTmaX) cp_async_wait_all();   // (nothing in flight when the shared memory goes away)
-  } else if (warp == 2 || warp == kEpiWarp0 + kEpiWarps) {
+  } else if (warp == 2 || warp == kMma1) {
     // ------------------------------------------------------------------ MMA issue
     // A warp cannot run ahead of the tensor cores by more than an MMA or two, so everything it does between
     // two groups of MMAs - barriers polled, commits (the second of a pair alone 73 cycles), the loop - adds
@@ -689,7 +691,7 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
     // few sequences each.
     const uint32_t et = tid - kEpiWarp0 * 32, quarter = warp & 3u, hh = (warp - kEpiWarp0) >> 2;
     const uint32_t l128 = quarter * 32u + lane;   // tensor-memory lane
-    uint32_t as = 0, apar = 0, n_xch = 0;
+    uint32_t as = 0, apar = 0, n_xch = 0, n_free = 0;
     pdl_wait();
     const uint32_t skip = et == 0 ? skip_arrivals_of(p.ws) : 0u;
     for (uint32_t ph = 0; ph < p.n_phases; ++ph) {
@@ -782,8 +784,8 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
           }
         }
       };
-      // Finish columns [0, cols) = sequences [mb, mb + cols) of an image: own sums, the peer's sums (or null).  aux of the first G columns is loaded.
-      auto finish = [&](const float* own, const float* in, uint32_t mb, uint32_t cols, uint32_t image_no) {
+      // Finish columns [0, cols) = sequences [mb, mb + cols) of an image: own sums, the peer's sums (or null; a column in_lanes apart).  aux of the first G columns is loaded.
+      auto finish = [&](const float* own, const float* in, uint32_t in_lanes, uint32_t mb, uint32_t cols, uint32_t image_no) {
         for (uint32_t i0 = 0; i0 * m_step < cols; i0 += G) {   // G at a time, so that their loads and arithmetic overlap
           if (i0) load_aux(mb, cols, i0);
           float lo[G], hi[G];
@@ -795,8 +797,9 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
             lo[g] = own[at];
             hi[g] = own[at + n_pos];
             if (in) {
-              lo[g] += in[at];
-              hi[g] += in[at + n_pos];
+              const float* const peer = in + (c < cols ? c : 0u) * in_lanes + pos;
+              lo[g] += peer[0];
+              hi[g] += peer[n_pos];
             }
           }
           const uint32_t m0 = mb + col + i0 * m_step;
@@ -1046,32 +1049,34 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
           const uint32_t half = nb / 2 / kRounds;                             // columns of a round that one threadblock finishes
           const uint32_t lanes = m64 ? 64u : kRowTile;                        // that hold sums
           float* own = kBig ? reinterpret_cast<float*>(x_ring) : sums;
-          float* in = own + half * kRowTile;
+          // At 64 and 128 rows the peer's sums arrive in the chunk buffer, idle here, where they fit; else in the activation slots,
+          // once this threadblock's products have read them, which the peer is told (a microsecond: down product at
+          // batch 64 / 128 25.2 -> 24.2, 30.3 -> 29.3 us without).
+          const bool roomy = !kBig || (kRounds == 1 && half * lanes * 4u <= sums_bytes(kN));
+          const uint32_t in_lanes = kBig && kRounds == 1 ? lanes : kRowTile;
+          float* in = kBig && roomy ? sums : own + half * kRowTile;
           place(w.u0);
           if (epi == BOOST_EPI_ROPE_APPEND) row_table();
-          // (from 128 rows on these operands wait in the chunk buffer, idle here, so that all rounds' are asked
-          // for ahead of the sums: about 1 % of a step)
-          float* const kept = sums + et;
+          // (At 256 rows these operands wait in the chunk buffer, so that all rounds' are asked for ahead of the sums: about 1 % of a step.)
+          [[maybe_unused]] float* const kept = sums + et;
 #pragma unroll
-          for (uint32_t r = 0; r < (kParkSums ? kRounds : 1); ++r) {
+          for (uint32_t r = 0; r < kRounds; ++r) {
             load_aux((2 * r + rank) * half, half, 0);
-            if constexpr (kParkSums)
+            if constexpr (kRounds > 1)
 #pragma unroll
               for (uint32_t g = 0; g < G; ++g) {
                 kept[((r * G + g) * 2) * kEpiThreads] = aux_a[g];
                 kept[((r * G + g) * 2 + 1) * kEpiThreads] = aux_b[g];
               }
           }
-          if constexpr (!kBig)
-            if (et == 0) mbar_arrive_expect_tx(&xch_full, lanes * half * 4u);
+          if (et == 0) mbar_arrive_expect_tx(&xch_full, lanes * half * kRounds * 4u);
           accumulate();
-          if constexpr (kBig) {
-            // the peer may store here once this threadblock's products have read the activation slots
+          if (!roomy) {
             if (et == 0) {
-              mbar_arrive_expect_tx(&xch_full, lanes * half * kRounds * 4u);
               arrive_remote(mapa(smem_u32(&xch_free), rank ^ 1u));
-              wait(smem_u32(&xch_free), n_xch & 1u);
+              wait(smem_u32(&xch_free), n_free & 1u);
             }
+            ++n_free;
             named_barrier_sync(1, kEpiThreads);
           }
           if (!__any_sync(0xFFFFFFFFu, s_abort != 0)) {   // the peer's columns, of all rounds
@@ -1084,13 +1089,13 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
               group_sums(i, v);
               if (holds) {
 #pragma unroll
-                for (uint32_t e = 0; e < CH; ++e) st_async_f32(to + ((c + e) * kRowTile + row) * 4u, v[e], bar);
+                for (uint32_t e = 0; e < CH; ++e) st_async_f32(to + ((c + e) * in_lanes + row) * 4u, v[e], bar);
               }
             }
           }
           for (uint32_t r = 0; r < kRounds; ++r) {
             const uint32_t mb = (2 * r + rank) * half;
-            if constexpr (kParkSums) {
+            if constexpr (kRounds > 1) {
 #pragma unroll
               for (uint32_t g = 0; g < G; ++g) {
                 aux_a[g] = kept[((r * G + g) * 2) * kEpiThreads];
@@ -1111,7 +1116,7 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
             if (kParkSums && r + 1 == kRounds) release_slot(parked);
             if (et == 0 && r == 0) wait(smem_u32(&xch_full), n_xch & 1u);
             named_barrier_sync(1, kEpiThreads);
-            finish(own, in + r * half * kRowTile, mb, half, 0);
+            finish(own, in + r * half * in_lanes, in_lanes, mb, half, 0);
             if constexpr (kBig) {
               fence_proxy_async_smem();   // (the activation slots are written by TMA copies again)
               named_barrier_sync(1, kEpiThreads);
@@ -1141,7 +1146,7 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
             }
             if (kParkSums && ch + 1 == n_chunks) release_slot(parked);
             named_barrier_sync(1, kEpiThreads);
-            finish(sums, nullptr, ch * CW, CW, image_no);
+            finish(sums, nullptr, 0, ch * CW, CW, image_no);
             named_barrier_sync(1, kEpiThreads);   // (the buffer and the row table are written again)
           }
         }
@@ -1167,21 +1172,22 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
     // may be in the tensor cores' pipeline or on its way to shared memory when that goes away.  Each
     // issuer waits, as long as any other wait, for what it has started.  (A fixed time would not do: over
     // the host link the copies in flight of all threadblocks are a third of a millisecond.)
-    if (warp == 2 || warp == kEpiWarp0 + kEpiWarps) {
+    if (warp == 2 || warp == kMma1) {
       uint64_t* const bar = &drained[warp == 2 ? 0 : 1];
       if (elect_one()) commit(smem_u32(bar));
       __syncwarp();
       mbar_wait(bar, 0, status);
-    } else if (warp < kEpiWarp0 && (warp != 1 || kTmaX)) {
+    } else if (warp == 0 || warp == 3 || (kTmaX && (warp == 1 || warp == kX1))) {
       // the last use of every stage, backwards from the next one (uses before the first count as landed)
-      const uint32_t n = warp == 1 ? pipe_slots : pipe_stages;
-      uint64_t* const full = warp == 1 ? x_full : w_full + (kPipes == 2 && warp == 3 ? pipe_stages : 0);
+      const bool weights = warp == 0 || warp == 3, second = kPipes == 2 && (warp == 3 || warp == kX1);
+      const uint32_t n = weights ? pipe_stages : pipe_slots;
+      uint64_t* const full = (weights ? w_full : x_full) + (second ? n : 0);
       for (uint32_t i = 0; i < n; ++i) {
         if (stage == 0) { stage = n; parity ^= 1u; }
         --stage;
-        if (kPipes == 1 && warp != 1) my_turn = !my_turn;
+        if (kPipes == 1 && weights) my_turn = !my_turn;
         if (my_turn) mbar_wait(full + stage, parity ^ 1u, status);
-        if (kPipes == 2 && warp == 1) {
+        if (kPipes == 2 && x_warps(kN) == 1 && !weights) {
           if (stage1 == 0) { stage1 = n; parity1 ^= 1u; }
           --stage1;
           mbar_wait(full + n + stage1, parity1 ^ 1u, status);
