@@ -86,6 +86,7 @@ struct PairPhase {
 
 struct PairParams {
   uint32_t n_phases, M_b, nb, n_stages, x_slots;   // nb: activation rows of a tile (the batch rounded up)
+  uint32_t chunk;  // columns of a chunk at 256 rows (see chunk_at)
   uint32_t early;  // weights and their page tables may be read while the kernel ahead on the stream still runs
   uint32_t* ws;    // workspace header
   uint32_t* bar;   // [0] threadblocks past their last wait, [1] phases finished, summed over the threadblocks; zero at rest
@@ -129,10 +130,14 @@ __host__ __device__ constexpr uint32_t x_warps(uint32_t n) { return n == 128 ? 2
 __host__ __device__ constexpr uint32_t epi_warps(uint32_t n) { return n <= 32 ? 8 : 16; }
 __host__ __device__ constexpr uint32_t threads_of(uint32_t n) { return (kEpiWarp0 + epi_warps(n) + pipes_of(n) - 1 + x_warps(n) - 1) * 32; }
 // Sums on their way from tensor memory to the threads that finish them, fp32 [columns][128 lanes].
-// Rows of one threadblock: this many columns at a time (32 in two buffers in turn were 1.5 % slower than 64
+// Rows of one threadblock: at most this many columns at a time (32 in two buffers in turn were 1.5 % slower than 64
 // for a step at batch 250).  128 rows: 32, so that shared memory holds six stages and six activation slots
-// (6-layer step at batch 128: 1503 us; 64 columns with six stages and four slots 1584, with four and six 1605).
+// (6-layer step at batch 128: 1477 us; six and four 1569, four and eight 1600).  256 rows: see chunk_at.
 __host__ __device__ constexpr uint32_t chunk_cols(uint32_t n) { return n < 64 ? n : n == 128 ? 32 : 64; }
+// 129 - 256 rows, tiles of nb rows: shared memory is short of activation slots, and four of 224 or 256 rows leave
+// room for 32 columns.  6-layer step, three slots and 64 columns -> four and 32: batch 200 1767 -> 1615 us, 250 1907 -> 1820.
+// Where four fit beside 64 columns that is better (batch 180 1518, with 32 and a stage more 1540).
+__host__ __device__ constexpr uint32_t chunk_at(uint32_t nb) { return nb <= 192 ? 64 : 32; }
 // Rows that two threadblocks share: each finishes half of the columns, in this many rounds.  The
 // columns of a round, this threadblock's sums and the peer's, are kept in the chunk buffers
 // (up to 32 rows), or this threadblock's in the activation slots, which are idle then, and the peer's in the
@@ -314,7 +319,8 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
   constexpr bool kTmaX = x_by_tma(kN);
   constexpr uint32_t kEpiWarps = epi_warps(kN), kEpiThreads = kEpiWarps * 32;
   constexpr bool kBig = kN >= 64;
-  constexpr uint32_t CW = chunk_cols(kN), CH = kBig ? 8 : kN / 2, HG = kEpiWarps / 4;   // columns of a chunk; of a group; warps that share lanes
+  const uint32_t CW = kN == 256 ? p.chunk : chunk_cols(kN);
+  constexpr uint32_t CH = kBig ? 8 : kN / 2, HG = kEpiWarps / 4;   // columns of a group; warps that share lanes
   extern __shared__ uint8_t smem_raw[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t n_stages = p.n_stages, x_slots = p.x_slots;
@@ -725,7 +731,7 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
       }
       // This thread's place: row `pos` of the image's lower (and upper) half, columns col, col + m_step, ... of a chunk or round
       const uint32_t n_pos = 4 * image, pos = et % n_pos, m_step = kEpiThreads / n_pos, col = et / n_pos;
-      constexpr uint32_t G = kBig ? 4 : CW / 8;                                      // columns a thread finishes at a time
+      constexpr uint32_t G = kBig ? 4 : kN / 8;                                      // columns a thread finishes at a time
       uint32_t ua, ub, u, d, n;   // the image: its run of units; the unit that sits at this position, and its rows of the weight
       bool valid;
       auto place = [&](uint32_t first) {
@@ -1057,17 +1063,13 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
           float* in = kBig && roomy ? sums : own + half * kRowTile;
           place(w.u0);
           if (epi == BOOST_EPI_ROPE_APPEND) row_table();
-          // (At 256 rows these operands wait in the chunk buffer, so that all rounds' are asked for ahead of the sums: about 1 % of a step.)
-          [[maybe_unused]] float* const kept = sums + et;
+          // (All rounds' operands are asked for ahead of the sums: about 1 % of a step.)
+          float kept_a[kRounds][G], kept_b[kRounds][G];
 #pragma unroll
           for (uint32_t r = 0; r < kRounds; ++r) {
             load_aux((2 * r + rank) * half, half, 0);
-            if constexpr (kRounds > 1)
 #pragma unroll
-              for (uint32_t g = 0; g < G; ++g) {
-                kept[((r * G + g) * 2) * kEpiThreads] = aux_a[g];
-                kept[((r * G + g) * 2 + 1) * kEpiThreads] = aux_b[g];
-              }
+            for (uint32_t g = 0; g < G; ++g) { kept_a[r][g] = aux_a[g]; kept_b[r][g] = aux_b[g]; }
           }
           if (et == 0) mbar_arrive_expect_tx(&xch_full, lanes * half * kRounds * 4u);
           accumulate();
@@ -1095,12 +1097,10 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
           }
           for (uint32_t r = 0; r < kRounds; ++r) {
             const uint32_t mb = (2 * r + rank) * half;
-            if constexpr (kRounds > 1) {
 #pragma unroll
-              for (uint32_t g = 0; g < G; ++g) {
-                aux_a[g] = kept[((r * G + g) * 2) * kEpiThreads];
-                aux_b[g] = kept[((r * G + g) * 2 + 1) * kEpiThreads];
-              }
+            for (uint32_t g = 0; g < G; ++g) {
+              aux_a[g] = r ? kept_a[kRounds - 1][g] : kept_a[0][g];
+              aux_b[g] = r ? kept_b[kRounds - 1][g] : kept_b[0][g];
             }
 #pragma unroll
             for (uint32_t i = 0; i < kGroups; ++i) {   // this threadblock's columns of the round
@@ -1126,7 +1126,8 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
           image_no = 1;
         }
       } else {
-        constexpr uint32_t J = CW / (HG * CH);   // groups of a chunk
+        constexpr uint32_t kChunkGroups = chunk_cols(kN) / (HG * CH);   // groups of a chunk, at most
+        const uint32_t J = CW / (HG * CH);
         const uint32_t n_chunks = (M_b + CW - 1) / CW;
         for (uint32_t ua0 = w.u0; ua0 < w.u1; ua0 += w.run, ++image_no) {
           place(ua0);
@@ -1136,7 +1137,8 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
           for (uint32_t ch = 0; ch < n_chunks; ++ch) {
             if (ch) load_aux(ch * CW, CW, 0);
 #pragma unroll
-            for (uint32_t j = 0; j < J; ++j) {
+            for (uint32_t j = 0; j < kChunkGroups; ++j) {
+              if (kN == 256 && j >= J) break;
               float v[CH];
               group_sums(kParkSums ? ch * J + j : j, v);   // (not parked: there is one chunk)
               if (holds) {
@@ -1306,12 +1308,14 @@ int launch_pair(PairParams& p, float* stats, size_t stats_bytes, cudaStream_t st
   if (rc != BOOST_OK) return rc;
   if (clusters == 0) return BOOST_ERR_UNSUPPORTED;
   // activation slots: more than a microsecond of a short product's stream (a k block per 155 ns); from
-  // 128 rows on about half of the shared memory, since the tiles are as large as the weight stages
+  // 128 rows on half of the shared memory and more, since the tiles are as large as the weight stages.  Above 128 rows
+  // four tiles, five where that leaves five stages (batch 150: 1431 -> 1388 us for 6 layers; 180: four 1518, five 1550).
   const uint32_t slot_bytes = x_blocks(kN) * p.nb * 128u;
-  const uint32_t x_budget = kN <= 16 ? 6 * slot_bytes : kN == 32 ? 4 * slot_bytes : kN == 64 ? 64u * 1024u : 96u * 1024u;
+  const uint32_t x_budget = kN <= 16 ? 6 * slot_bytes : kN == 32 ? 4 * slot_bytes : kN == 64 ? 64u * 1024u : kN == 128 ? 96u * 1024u : (p.nb <= 160 ? 5 : 4) * slot_bytes;
   p.x_slots = x_budget / slot_bytes < kMaxXSlots ? x_budget / slot_bytes : kMaxXSlots;
   p.x_slots = p.x_slots / pipes_of(kN) * pipes_of(kN);
-  const uint32_t fixed = 2048u + p.x_slots * slot_bytes + sums_bytes(kN);
+  p.chunk = kN == 256 ? chunk_at(p.nb) : chunk_cols(kN);
+  const uint32_t fixed = 2048u + p.x_slots * slot_bytes + (kN == 256 ? p.chunk * kRowTile * 4u : sums_bytes(kN));
   p.n_stages = (smem_total(kN) - fixed) / kStageBytes;
   if (p.n_stages > kMaxStages) p.n_stages = kMaxStages;
   p.n_stages = p.n_stages / pipes_of(kN) * pipes_of(kN);
