@@ -346,6 +346,21 @@ def test_gemv_at_the_edges_of_the_kernel_rule(dev, n, k, m_b):
     assert w.status_words() == [0]
 
 
+@pytest.mark.parametrize("n,k,m_b", [
+    (1001, 1088, 5), (1001, 1216, 24), (9601, 1088, 16), (1001, 1216, 70), (9601, 1088, 128),   # chunks of two k blocks: an odd last one, an odd number of them
+    (1001, 1152, 160), (9601, 1088, 161), (1001, 1088, 192), (9601, 1216, 193), (1001, 1216, 224), (9601, 1088, 225)])   # sizes of an activation tile
+def test_gemv_pipelines_and_tile_sizes(dev, n, k, m_b):
+    """The cluster kernel's two pipelines take chunks of k blocks in turn (8 - 19 blocks per threadblock here),
+    and from 129 rows on the size of an activation tile decides how many there are: against the
+    oracle, and every launch gives the same bits."""
+    w, y, ref, (x, res) = run_gemv(dev, n, k, m_b, 0.0, seed=n + k + m_b, residual=True)
+    assert_close_to_oracle(y, ref, f"{n} x {k}, batch {m_b}")
+    again = [w.gemv(x, residual=res) for _ in range(20)]
+    torch.cuda.synchronize()
+    assert all(np.array_equal(a.cpu().numpy(), y) for a in again)
+    assert w.status_words() == [0]
+
+
 @pytest.mark.parametrize("n,k,m_b", [(28672, 4096, 64), (4096, 4096, 256), (4096, 4096, 24), (6144, 4096, 7)])
 def test_split_k_kernels_at_full_size(dev, n, k, m_b):
     """The kernels whose partial sums meet in L2 at the sizes that plain products now take to the cluster kernel:
