@@ -475,12 +475,12 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
     };
     for (uint32_t ph = 0; ph < p.n_phases; ++ph)
       if (!produce(p.ph[ph], ph)) break;
-  } else if (warp == 1 || warp == kX1) {
+  } else if (warp == 1 || (x_warps(kN) == 2 && warp == kX1)) {
     // ------------------------------------------------------------------ activation producers
     // Up to 32 rows: 16-byte copies through the load/store path (the TMA unit works in order, and an
     // activation tile would queue behind the weight copies of a full ring).  Rows beyond the batch are
     // left as they are: they only reach accumulator columns that nobody reads.
-    const uint32_t pipe = warp == 1 ? 0u : 1u;
+    const uint32_t pipe = x_warps(kN) == 1 || warp == 1 ? 0u : 1u;
     const uint32_t x_a = smem_u32(x_ring), full_a = smem_u32(x_full), empty_a = smem_u32(x_empty);
     if constexpr (kTmaX) {
       if (elect_one())
@@ -506,8 +506,19 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
           for (uint32_t k0 = w.kb0; k0 < w.kb1; k0 += slot_n) {
             const uint32_t k1 = min(k0 + slot_n, w.kb1);
             for (uint32_t c = k0 + pipe * chunk; c < k1; c += 2 * chunk) {
+              if constexpr (kXB == 2) {   // a chunk is a slot
+                if (!wait(empty_a + stage * 8, parity)) return false;
+                fill(c, stage);
+                if (++stage == pipe_slots) { stage = 0; parity ^= 1u; }
+                if (c + 2 < k1) {
+                  if (!wait(empty_a + (pipe_slots + stage1) * 8, parity1)) return false;
+                  fill(c + 2, pipe_slots + stage1);
+                  if (++stage1 == pipe_slots) { stage1 = 0; parity1 ^= 1u; }
+                }
+              } else {
               if (!put(c, min(c + chunk, k1), pipe * pipe_slots, stage, parity)) return false;
               if (x_warps(kN) == 1 && !put(c + chunk, min(c + 2 * chunk, k1), pipe_slots, stage1, parity1)) return false;
+              }
             }
           }
         }
@@ -563,7 +574,7 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
     for (uint32_t ph = 0; ph < p.n_phases; ++ph) {
       if (ph > 0) {
         // one lane polls; the barrier orders the other lanes' reads behind what it has acquired
-        if (pipe) wait(smem_u32(&go), (ph - 1) & 1u);
+        if (x_warps(kN) == 2 && pipe) wait(smem_u32(&go), (ph - 1) & 1u);
         else if (lane == 0) {
           if (!s_abort && !grid_counter_wait(p.bar + 1, ph * n_cta, status)) s_abort = 1;
           mbar_arrive(&go);   // the epilogue warps (and the second producer) may read what the phase before wrote
@@ -803,9 +814,14 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
             lo[g] = own[at];
             hi[g] = own[at + n_pos];
             if (in) {
-              const float* const peer = in + (c < cols ? c : 0u) * in_lanes + pos;
-              lo[g] += peer[0];
-              hi[g] += peer[n_pos];
+              if constexpr (kBig) {
+                const float* const peer = in + (c < cols ? c : 0u) * in_lanes + pos;
+                lo[g] += peer[0];
+                hi[g] += peer[n_pos];
+              } else {
+                lo[g] += in[at];
+                hi[g] += in[at + n_pos];
+              }
             }
           }
           const uint32_t m0 = mb + col + i0 * m_step;
