@@ -330,7 +330,11 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
   // (an 8-row activation tile is read as 16 rows: 1 KiB behind the slots)
   float* sums = reinterpret_cast<float*>(x_ring + x_slot * x_slots + 1024u);
   __shared__ uint64_t w_full[kMaxStages], w_empty[kMaxStages], x_full[kMaxXSlots], x_empty[kMaxXSlots];
-  __shared__ uint64_t acc_full[kMaxAccSlots], acc_empty[kMaxAccSlots], xch_full, xch_free, go, drained[2];
+  __shared__ uint64_t acc_full[kMaxAccSlots], acc_empty[kMaxAccSlots], xch_full, xch_free, drained[2];
+  // The phases after the first may start.  One barrier each: a second activation producer that fills no slot of a
+  // phase holds nobody up in it, so its look at one barrier for all could come after the next phase's arrival, where the
+  // parity reads as not arrived yet and the wait would not end.
+  __shared__ uint64_t go[kMaxPhases - 1];
   __shared__ uint32_t s_tmem;
   __shared__ uint32_t s_rec[kMaxPhases];
   __shared__ float s_rs[kN], s_red[kEpiThreads];
@@ -354,7 +358,7 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
     }
     mbar_init(&xch_full, 1);
     mbar_init(&xch_free, 1);
-    mbar_init(&go, 1);
+    for (uint32_t i = 0; i < kMaxPhases - 1; ++i) mbar_init(&go[i], 1);
     mbar_init(&drained[0], 1);
     mbar_init(&drained[1], 1);
     s_abort = 0;
@@ -574,10 +578,10 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
     for (uint32_t ph = 0; ph < p.n_phases; ++ph) {
       if (ph > 0) {
         // one lane polls; the barrier orders the other lanes' reads behind what it has acquired
-        if (x_warps(kN) == 2 && pipe) wait(smem_u32(&go), (ph - 1) & 1u);
+        if (x_warps(kN) == 2 && pipe) wait(smem_u32(&go[ph - 1]), 0);
         else if (lane == 0) {
           if (!s_abort && !grid_counter_wait(p.bar + 1, ph * n_cta, status)) s_abort = 1;
-          mbar_arrive(&go);   // the epilogue warps (and the second producer) may read what the phase before wrote
+          mbar_arrive(&go[ph - 1]);   // the epilogue warps (and the second producer) may read what the phase before wrote
           // The last threadblock past the last of these waits - everybody has arrived, nobody reads the
           // counters any more - puts them back to zero for the next launch.  (Here and not at the end of
           // the kernel, where the round trip would hold up the kernel that waits for this one.)
@@ -718,7 +722,7 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
       const uint32_t image = q.image, worker = two ? blockIdx.x >> 1 : blockIdx.x;
       const uint32_t epi = q.epi, N = q.N, M_b = p.M_b;
       if (ph > 0) {   // (one thread polls, the others wait in the hardware barrier)
-        if (et == 0) wait(smem_u32(&go), (ph - 1) & 1u);
+        if (et == 0) wait(smem_u32(&go[ph - 1]), 0);
         // After a wait that gave up, everybody leaves before the next phase: a barrier whose peer never
         // came is not armed a second time.
         if (named_barrier_or(1, kEpiThreads, s_abort != 0)) break;
