@@ -86,7 +86,6 @@ struct PairPhase {
 
 struct PairParams {
   uint32_t n_phases, M_b, nb, n_stages, x_slots;   // nb: activation rows of a tile (the batch rounded up)
-  uint32_t chunk;  // columns of a chunk at 256 rows (see chunk_at)
   uint32_t early;  // weights and their page tables may be read while the kernel ahead on the stream still runs
   uint32_t* ws;    // workspace header
   uint32_t* bar;   // [0] threadblocks past their last wait, [1] phases finished, summed over the threadblocks; zero at rest
@@ -132,18 +131,14 @@ __host__ __device__ constexpr uint32_t threads_of(uint32_t n) { return (kEpiWarp
 // Sums on their way from tensor memory to the threads that finish them, fp32 [columns][128 lanes].
 // Rows of one threadblock: at most this many columns at a time (32 in two buffers in turn were 1.5 % slower than 64
 // for a step at batch 250).  128 rows: 32, so that shared memory holds six stages and six activation slots
-// (6-layer step at batch 128: 1477 us; six and four 1569, four and eight 1600).  256 rows: see chunk_at.
-__host__ __device__ constexpr uint32_t chunk_cols(uint32_t n) { return n < 64 ? n : n == 128 ? 32 : 64; }
-// 129 - 256 rows, tiles of nb rows: shared memory is short of activation slots, and four of 224 or 256 rows leave
-// room for 32 columns.  6-layer step, three slots and 64 columns -> four and 32: batch 200 1767 -> 1615 us, 250 1907 -> 1820.
-// Where four fit beside 64 columns that is better (batch 180 1518, with 32 and a stage more 1540).
-__host__ __device__ constexpr uint32_t chunk_at(uint32_t nb) { return nb <= 192 ? 64 : 32; }
+// (6-layer step at batch 128: 1477 us; six and four 1569, four and eight 1600).  256 rows: 64 or 32 (see wide_chunk).
+[[maybe_unused]] __host__ __device__ constexpr uint32_t chunk_cols(uint32_t n) { return n < 64 ? n : n == 128 ? 32 : 64; }
 // Rows that two threadblocks share: each finishes half of the columns, in this many rounds.  The
 // columns of a round, this threadblock's sums and the peer's, are kept in the chunk buffers
 // (up to 32 rows), or this threadblock's in the activation slots, which are idle then, and the peer's in the
 // chunk buffer where they fit (64 and 128 rows).
 __host__ __device__ constexpr uint32_t rounds_of(uint32_t n) { return n >= 256 ? 2 : 1; }
-__host__ __device__ constexpr uint32_t sums_bytes(uint32_t n) { return chunk_cols(n) * kRowTile * 4; }
+__host__ __device__ constexpr uint32_t sums_bytes(uint32_t chunk) { return chunk * kRowTile * 4; }
 
 template <auto kValue>
 struct Const { static constexpr auto value = kValue; };
@@ -313,14 +308,13 @@ __device__ __noinline__ uint32_t host_bytes_of_range(const PairPhase& q, uint32_
   return bytes;
 }
 
-template <uint32_t kN>
+template <uint32_t kN, uint32_t kChunk>
 __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_constant__ PairParams p) {
   constexpr uint32_t kXB = x_blocks(kN), kSlots = acc_slots(kN), kSlotCols = slot_cols(kN), kPipes = pipes_of(kN);
   constexpr bool kTmaX = x_by_tma(kN);
   constexpr uint32_t kEpiWarps = epi_warps(kN), kEpiThreads = kEpiWarps * 32;
   constexpr bool kBig = kN >= 64;
-  const uint32_t CW = kN == 256 ? p.chunk : chunk_cols(kN);
-  constexpr uint32_t CH = kBig ? 8 : kN / 2, HG = kEpiWarps / 4;   // columns of a group; warps that share lanes
+  constexpr uint32_t CW = kChunk, CH = kBig ? 8 : kN / 2, HG = kEpiWarps / 4;   // columns of a group; warps that share lanes
   extern __shared__ uint8_t smem_raw[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t n_stages = p.n_stages, x_slots = p.x_slots;
@@ -1078,19 +1072,21 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
           // At 64 and 128 rows the peer's sums arrive in the chunk buffer, idle here, where they fit; else in the activation slots,
           // once this threadblock's products have read them, which the peer is told (a microsecond: down product at
           // batch 64 / 128 25.2 -> 24.2, 30.3 -> 29.3 us without).
-          const bool roomy = !kBig || (kRounds == 1 && half * lanes * 4u <= sums_bytes(kN));
+          const bool roomy = !kBig || (kRounds == 1 && half * lanes * 4u <= sums_bytes(CW));
           const uint32_t in_lanes = kBig && kRounds == 1 ? lanes : kRowTile;
           float* in = kBig && roomy ? sums : own + half * kRowTile;
           place(w.u0);
           if (epi == BOOST_EPI_ROPE_APPEND) row_table();
-          // (All rounds' operands are asked for ahead of the sums: about 1 % of a step.)
-          float kept_a[kRounds][G], kept_b[kRounds][G];
+          // (All rounds' operands are asked for ahead of the sums: about 1 % of a step.  A second round's wait in the chunk
+          // buffer, idle here: in registers, which are short above 128 rows, they cost products of few k blocks 1 - 2 %.)
+          float* const kept = sums + et;
+          static_assert(kRounds == 1 || 2 * G * kEpiThreads <= CW * kRowTile, "operands fit the chunk buffer");
+          if constexpr (kRounds == 2) {
+            load_aux((2 + rank) * half, half, 0);
 #pragma unroll
-          for (uint32_t r = 0; r < kRounds; ++r) {
-            load_aux((2 * r + rank) * half, half, 0);
-#pragma unroll
-            for (uint32_t g = 0; g < G; ++g) { kept_a[r][g] = aux_a[g]; kept_b[r][g] = aux_b[g]; }
+            for (uint32_t g = 0; g < G; ++g) { kept[2 * g * kEpiThreads] = aux_a[g]; kept[(2 * g + 1) * kEpiThreads] = aux_b[g]; }
           }
+          load_aux(rank * half, half, 0);
           if (et == 0) mbar_arrive_expect_tx(&xch_full, lanes * half * kRounds * 4u);
           accumulate();
           if (!roomy) {
@@ -1117,10 +1113,9 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
           }
           for (uint32_t r = 0; r < kRounds; ++r) {
             const uint32_t mb = (2 * r + rank) * half;
+            if (kRounds == 2 && r == 1) {
 #pragma unroll
-            for (uint32_t g = 0; g < G; ++g) {
-              aux_a[g] = r ? kept_a[kRounds - 1][g] : kept_a[0][g];
-              aux_b[g] = r ? kept_b[kRounds - 1][g] : kept_b[0][g];
+              for (uint32_t g = 0; g < G; ++g) { aux_a[g] = kept[2 * g * kEpiThreads]; aux_b[g] = kept[(2 * g + 1) * kEpiThreads]; }
             }
 #pragma unroll
             for (uint32_t i = 0; i < kGroups; ++i) {   // this threadblock's columns of the round
@@ -1146,8 +1141,7 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
           image_no = 1;
         }
       } else {
-        constexpr uint32_t kChunkGroups = chunk_cols(kN) / (HG * CH);   // groups of a chunk, at most
-        const uint32_t J = CW / (HG * CH);
+        constexpr uint32_t J = CW / (HG * CH);   // groups of a chunk
         const uint32_t n_chunks = (M_b + CW - 1) / CW;
         for (uint32_t ua0 = w.u0; ua0 < w.u1; ua0 += w.run, ++image_no) {
           place(ua0);
@@ -1157,8 +1151,7 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
           for (uint32_t ch = 0; ch < n_chunks; ++ch) {
             if (ch) load_aux(ch * CW, CW, 0);
 #pragma unroll
-            for (uint32_t j = 0; j < kChunkGroups; ++j) {
-              if (kN == 256 && j >= J) break;
+            for (uint32_t j = 0; j < J; ++j) {
               float v[CH];
               group_sums(kParkSums ? ch * J + j : j, v);   // (not parked: there is one chunk)
               if (holds) {
@@ -1272,7 +1265,7 @@ constexpr uint32_t smem_total(uint32_t n) { return (n <= 32 ? 147u : 214u) * 102
 
 // Clusters of two that the current device holds at once, one threadblock per SM (0: none, or an error, which
 // is left in `rc`).  Set up once per device; every rule about how a product is cut starts from here.
-template <uint32_t kN>
+template <uint32_t kN, uint32_t kChunk = chunk_cols(kN)>
 uint32_t clusters_of(int& rc) {
   static std::atomic<uint32_t> known[boosth::kMaxDevices];   // count + 1; threads that meet here find the same
   const int dev = boosth::device_slot(), sms = boosth::sm_count();
@@ -1280,7 +1273,7 @@ uint32_t clusters_of(int& rc) {
   if (rc != BOOST_OK) return 0;
   const uint32_t seen = known[dev].load(std::memory_order_acquire);
   if (seen) return seen - 1;
-  rc = boosth::check(cudaFuncSetAttribute(gemv_pair_kernel<kN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_total(kN)));
+  rc = boosth::check(cudaFuncSetAttribute(gemv_pair_kernel<kN, kChunk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_total(kN)));
   if (rc != BOOST_OK) return 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2);
@@ -1294,7 +1287,7 @@ uint32_t clusters_of(int& rc) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  rc = boosth::check(cudaOccupancyMaxActiveClusters(&n, gemv_pair_kernel<kN>, &cfg));
+  rc = boosth::check(cudaOccupancyMaxActiveClusters(&n, gemv_pair_kernel<kN, kChunk>, &cfg));
   if (rc != BOOST_OK) return 0;
   const uint32_t clusters = (uint32_t)n < (uint32_t)sms / 2 ? (uint32_t)n : (uint32_t)sms / 2;
   known[dev].store(clusters + 1, std::memory_order_release);
@@ -1319,23 +1312,48 @@ uint32_t clusters_for(uint32_t M_b) {
   return n ? n : 74;
 }
 
+// 129 - 256 rows: 64 columns to an epilogue's chunk, or 32?  Where four activation slots fit beside 64 that is better (tiles of
+// up to 192 rows: 6-layer step at batch 180 1518 us, with 32 and a stage more 1540).  Tiles of 224 rows: 32, and
+// a fourth slot in the room that leaves (batch 200: 1767 -> 1615).  Of 256 rows: the fourth slot pays where a product waits
+// for activations (batch 250: 1907 -> 1820), and 64 columns, with three slots, where rows that are one threadblock's
+// have few k blocks, so that the epilogue is most of its time.  Measured at batch 232 - 256, weights from HBM, by the
+// average number of blocks of 8 rows x 64 columns in an image.  Products on their own (9600 - 60000 rows x 1024 - 4096
+// columns): the times meet at 330 - 430 blocks for fp32 results, 390 - 460 for bf16, the lower ones where there is another
+// image, whose MMAs hide the epilogue (28672 x 1024, 194 blocks: 32 columns 30.6 us, 64 27.7; 14336 x 4096, 775: 41.5, 45.1).
+// Chains of a step: six models of 300 - 470 blocks 0 - 2 % faster with 64, one of 775 (the 8B model) 4 % with 32.
+bool wide_chunk(const PairParams& p) {
+  if (p.nb <= 224) return p.nb <= 192;
+  const uint32_t clusters = clusters_for(p.M_b);
+  bool wide = false;
+  for (uint32_t i = 0; i < p.n_phases; ++i) {
+    PairPhase q = p.ph[i];
+    plan_phase(q, clusters, 256, p.M_b);
+    if (q.split == 2) continue;
+    const bool fp32 = q.epi == BOOST_EPI_PLAIN && q.y_dtype == 0;
+    const uint32_t most = p.n_phases > 1 ? 500u : q.max_images > 1 ? (fp32 ? 330u : 390u) : fp32 ? 372u : 440u;
+    if ((uint64_t)q.n_units * q.k_blocks > (uint64_t)most * 2 * clusters * q.max_images) return false;
+    wide = true;
+  }
+  return wide;
+}
+
 // Row statistics between the phases of one launch live in two buffers of the workspace; a phase's
 // ssq_in is matched to the earlier phase that produces it by the caller's ssq_out pointer.
-template <uint32_t kN>
+template <uint32_t kN, uint32_t kChunk = chunk_cols(kN)>
 int launch_pair(PairParams& p, float* stats, size_t stats_bytes, cudaStream_t stream) {
   int rc;
-  const uint32_t clusters = clusters_of<kN>(rc);
+  const uint32_t clusters = clusters_of<kN, kChunk>(rc);
   if (rc != BOOST_OK) return rc;
   if (clusters == 0) return BOOST_ERR_UNSUPPORTED;
   // activation slots: more than a microsecond of a short product's stream (a k block per 155 ns); from
   // 128 rows on half of the shared memory and more, since the tiles are as large as the weight stages.  Above 128 rows
-  // four tiles, five where that leaves five stages (batch 150: 1431 -> 1388 us for 6 layers; 180: four 1518, five 1550).
+  // four tiles, five where that leaves five stages (batch 150: 1431 -> 1388 us for 6 layers; 180: four 1518, five 1550), and
+  // of 256 rows three where the chunks have 64 columns.
   const uint32_t slot_bytes = x_blocks(kN) * p.nb * 128u;
-  const uint32_t x_budget = kN <= 16 ? 6 * slot_bytes : kN == 32 ? 4 * slot_bytes : kN == 64 ? 64u * 1024u : kN == 128 ? 96u * 1024u : (p.nb <= 160 ? 5 : 4) * slot_bytes;
+  const uint32_t x_budget = kN <= 16 ? 6 * slot_bytes : kN == 32 ? 4 * slot_bytes : kN == 64 ? 64u * 1024u : kN == 128 ? 96u * 1024u : (p.nb <= 160 ? 5 : p.nb == 256 && kChunk == 64 ? 3 : 4) * slot_bytes;
   p.x_slots = x_budget / slot_bytes < kMaxXSlots ? x_budget / slot_bytes : kMaxXSlots;
   p.x_slots = p.x_slots / pipes_of(kN) * pipes_of(kN);
-  p.chunk = kN == 256 ? chunk_at(p.nb) : chunk_cols(kN);
-  const uint32_t fixed = 2048u + p.x_slots * slot_bytes + (kN == 256 ? p.chunk * kRowTile * 4u : sums_bytes(kN));
+  const uint32_t fixed = 2048u + p.x_slots * slot_bytes + sums_bytes(kChunk);
   p.n_stages = (smem_total(kN) - fixed) / kStageBytes;
   if (p.n_stages > kMaxStages) p.n_stages = kMaxStages;
   p.n_stages = p.n_stages / pipes_of(kN) * pipes_of(kN);
@@ -1360,7 +1378,7 @@ int launch_pair(PairParams& p, float* stats, size_t stats_bytes, cudaStream_t st
       q.ssq_out = stats + (n_stats++ & 1u) * (stats_bytes / 8);
     }
   }
-  return boosth::launch_chained_cluster(gemv_pair_kernel<kN>, dim3(2 * clusters), dim3(threads_of(kN)), smem, 2, stream, p);
+  return boosth::launch_chained_cluster(gemv_pair_kernel<kN, kChunk>, dim3(2 * clusters), dim3(threads_of(kN)), smem, 2, stream, p);
 }
 
 }  // namespace
@@ -1451,6 +1469,6 @@ int boosth::gemv_pair_launch(const boost_gemv_call_t* calls, uint32_t n_calls, u
     case 32: return launch_pair<32>(p, stats, stats_bytes, st);
     case 64: return launch_pair<64>(p, stats, stats_bytes, st);
     case 128: return launch_pair<128>(p, stats, stats_bytes, st);
-    default: return launch_pair<256>(p, stats, stats_bytes, st);
+    default: return wide_chunk(p) ? launch_pair<256>(p, stats, stats_bytes, st) : launch_pair<256, 32>(p, stats, stats_bytes, st);
   }
 }
