@@ -121,6 +121,11 @@ __host__ __device__ constexpr uint32_t tmem_cols(uint32_t n) { return acc_slots(
 __host__ __device__ constexpr uint32_t chunk_blocks(uint32_t n, uint32_t image) {
   return pipes_of(n) == 1 ? 1 : image == 8 || x_blocks(n) == 2 ? 2 : 1;
 }
+// Slots of one chunk go to the pipelines in turn.  (128 rows, images of 8, a k block to an accumulator.  All to the first pipeline,
+// half of the ring idle: fp32 results at batch 80, 1000 x 1024 10.65 us, 2048 x 1536 12.9; in turn 10.3, 12.5.)
+__host__ __device__ constexpr bool slots_in_turn(uint32_t n, uint32_t image, uint32_t slot_blocks) {
+  return n == 128 && slot_blocks == chunk_blocks(n, image);
+}
 // Activation producers.  (At 128 rows one is too slow for both pipelines: 375 cycles a slot, where the tensor cores take
 // 256 and HBM 275; down product 34.2 -> 30.2 us with two.  Fewer rows: slots of two blocks; batch 64 was 0.6 % slower with two.)
 __host__ __device__ constexpr uint32_t x_warps(uint32_t n) { return n == 128 ? 2 : 1; }
@@ -406,7 +411,7 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
     auto produce = [&](const PairPhase& q, uint32_t ph) -> bool {
       const Part w = part_of(q);
       const uint32_t image = q.image, k_blocks = q.k_blocks, n_pages = q.n_pages;
-      [[maybe_unused]] const uint32_t slot_n = q.slot_blocks, chunk = chunk_blocks(kN, image);
+      [[maybe_unused]] const uint32_t slot_n = q.slot_blocks, chunk = chunk_blocks(kN, image), in_turn = slots_in_turn(kN, image, slot_n);
       const void* const* const page_ptr = q.w_page_ptr;
       const bool twos = image == 8;
       if (warp == 0 && lane == 0) {
@@ -453,9 +458,10 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
         };
         auto next_stage = [&]() { if (++stage == pipe_stages) { stage = 0; parity ^= 1u; } };
         if constexpr (kPipes == 2) {
-          for (uint32_t k0 = w.kb0; k0 < w.kb1; k0 += slot_n) {
+          uint32_t turn = pipe;   // 0: the slot's first chunk
+          for (uint32_t k0 = w.kb0; k0 < w.kb1; k0 += slot_n, turn ^= in_turn) {
             const uint32_t k1 = min(k0 + slot_n, w.kb1);
-            for (uint32_t kb = k0 + pipe * chunk; kb < k1; kb += 2 * chunk)
+            for (uint32_t kb = k0 + turn * chunk; kb < k1; kb += 2 * chunk)
               for (uint32_t j = kb; j < min(kb + chunk, k1); j += step) {
                 if (!fill(j)) return false;
                 next_stage();
@@ -500,10 +506,11 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
         if constexpr (kPipes == 1) {
           if (!put(w.kb0, w.kb1, 0, stage, parity)) return false;
         } else {
-          const uint32_t chunk = chunk_blocks(kN, q.image), slot_n = q.slot_blocks;
-          for (uint32_t k0 = w.kb0; k0 < w.kb1; k0 += slot_n) {
+          const uint32_t chunk = chunk_blocks(kN, q.image), slot_n = q.slot_blocks, in_turn = slots_in_turn(kN, q.image, slot_n);
+          uint32_t turn = pipe;
+          for (uint32_t k0 = w.kb0; k0 < w.kb1; k0 += slot_n, turn ^= in_turn) {
             const uint32_t k1 = min(k0 + slot_n, w.kb1);
-            for (uint32_t c = k0 + pipe * chunk; c < k1; c += 2 * chunk) {
+            for (uint32_t c = k0 + turn * chunk; c < k1; c += 2 * chunk) {
               if constexpr (kXB == 2) {   // a chunk is a slot
                 if (!wait(empty_a + stage * 8, parity)) return false;
                 fill(c, stage);
@@ -630,7 +637,7 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
       constexpr uint32_t kStep = kPipes == 1 ? (kImage8 && kMode == 2 ? 2 : 1) : chunk_blocks(kN, kImage8 ? 8 : 16);
       constexpr bool kHalves = kImage8 && kStep == 1;
       const Part w = part_of(q);
-      const uint32_t slot_n = q.slot_blocks, id = kImage8 ? idesc64 : idesc;
+      const uint32_t slot_n = q.slot_blocks, id = kImage8 ? idesc64 : idesc, in_turn = kPipes == 2 && slots_in_turn(kN, kImage8 ? 8 : 16, slot_n);
       constexpr uint32_t kBlockCols = kMode == 2 ? 0 : kMode == 1 ? part_cols(kN) : 4 * part_cols(kN), kNext = kMode == 0 ? part_cols(kN) : 0;
       // One k block: 4 MMAs.  (16 columns on: 32 bytes, 2 in a descriptor's address field, which counts in 16 bytes)
       auto mma_block = [&](uint32_t d, uint32_t wl, uint32_t xl, uint32_t accumulate) {
@@ -639,11 +646,12 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
           umma_low(d + ks * kNext, wl + 2 * ks, xl + 2 * ks, id, kMode == 0 ? 0u : ks == 0 ? accumulate : 1u);
       };
       for (uint32_t ua = w.u0; ua < w.u1; ua += w.run) {
-        for (uint32_t k0 = w.kb0; k0 < w.kb1; k0 += slot_n) {   // a slot of accumulators: the epilogue warps have read what was there
+        uint32_t turn = pipe;
+        for (uint32_t k0 = w.kb0; k0 < w.kb1; k0 += slot_n, turn ^= in_turn) {   // a slot of accumulators: the epilogue warps have read what was there
           const uint32_t k1 = min(k0 + slot_n, w.kb1), done = afull_a + as * 8;
-          uint32_t d = tmem + as * kSlotCols + pipe * (kMode == 2 ? part_cols(kN) : kStep * kBlockCols), accumulate = 0;
+          uint32_t d = tmem + as * kSlotCols + turn * (kMode == 2 ? part_cols(kN) : kStep * kBlockCols), accumulate = 0;
           if (!wait_one(aempty_a + as * 8, apar)) return false;
-          for (uint32_t kb = k0 + pipe * kStep; kb < k1; kb += kPipes * kStep, d += kPipes * kStep * kBlockCols) {
+          for (uint32_t kb = k0 + turn * kStep; kb < k1; kb += kPipes * kStep, d += kPipes * kStep * kBlockCols) {
             const bool both = kStep == 2 && kb + 1 < k1, second = kHalves && ((kb - w.kb0) & 1u), last = !kHalves || second || kb + 1 == w.kb1;
             const uint32_t wl = w_low + stage * (kStageBytes / 16) + (second ? kStageBytes / 32 : 0u), xl = x_low + xs * x_step;
             const uint32_t free_w = empty_a + stage * 8, free_x = xempty_a + xs * 8;

@@ -348,6 +348,7 @@ def test_gemv_at_the_edges_of_the_kernel_rule(dev, n, k, m_b):
 
 @pytest.mark.parametrize("n,k,m_b", [
     (1001, 1088, 5), (1001, 1216, 24), (9601, 1088, 16), (1001, 1216, 70), (9601, 1088, 128),   # chunks of two k blocks: an odd last one, an odd number of them
+    (1001, 1032, 70), (2049, 1088, 80), (300, 1160, 100),   # ... one to a slot of accumulators
     (1001, 1152, 160), (9601, 1088, 161), (1001, 1088, 192), (9601, 1216, 193), (1001, 1216, 224), (9601, 1088, 225),   # sizes of an activation tile
     (9601, 2880, 241), (9601, 2944, 250), (19001, 2560, 250), (19001, 2624, 256)])   # 256-row tiles: three and four of them, one and two images
 def test_gemv_pipelines_and_tile_sizes(dev, n, k, m_b):
