@@ -313,8 +313,10 @@ __device__ __noinline__ uint32_t host_bytes_of_range(const PairPhase& q, uint32_
   return bytes;
 }
 
+// Registers: beside an attention threadblock (up to 32 rows) and within an SM (up to 128) as many as measured best: hidden
+// 256, 24 sequences with 80 77.1 us, with 96 75.8; 12 sequences with 80 66.1, with 88 65.1; 8B steps the same.
 template <uint32_t kN, uint32_t kChunk>
-__global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_constant__ PairParams p) {
+__global__ void __maxnreg__(kN >= 256 || kN == 32 ? 96 : kN == 16 ? 88 : 80) gemv_pair_kernel(const __grid_constant__ PairParams p) {
   constexpr uint32_t kXB = x_blocks(kN), kSlots = acc_slots(kN), kSlotCols = slot_cols(kN), kPipes = pipes_of(kN);
   constexpr bool kTmaX = x_by_tma(kN);
   constexpr uint32_t kEpiWarps = epi_warps(kN), kEpiThreads = kEpiWarps * 32;
@@ -348,19 +350,35 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
   const uint32_t n_cta = gridDim.x;
 
   pdl_launch_dependents();
-  if (tid == 0) {
-    for (uint32_t s = 0; s < n_stages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); }
-    for (uint32_t s = 0; s < x_slots; ++s) { mbar_init(&x_full[s], kTmaX ? 1 : 32); mbar_init(&x_empty[s], 1); }
-    for (uint32_t s = 0; s < kSlots; ++s) {
-      mbar_init(&acc_full[s], kPipes);
-      mbar_init(&acc_empty[s], kEpiWarps);
+  auto init_stage = [&](uint32_t s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); };
+  auto init_x = [&](uint32_t s) { mbar_init(&x_full[s], kTmaX ? 1 : 32); mbar_init(&x_empty[s], 1); };
+  auto init_acc = [&](uint32_t s) { mbar_init(&acc_full[s], kPipes); mbar_init(&acc_empty[s], kEpiWarps); };
+  // A lane per barrier (one thread for all 40: short products up to 0.2 us slower).  32 rows: one thread (6-layer 8B steps of
+  // 20 / 24 / 32 sequences 896 / 923 / 979 us, with a lane each 899 / 929 / 982).
+  if constexpr (kN == 32) {
+    if (tid == 0) {
+      for (uint32_t s = 0; s < n_stages; ++s) init_stage(s);
+      for (uint32_t s = 0; s < x_slots; ++s) init_x(s);
+      for (uint32_t s = 0; s < kSlots; ++s) init_acc(s);
+      mbar_init(&xch_full, 1);
+      mbar_init(&xch_free, 1);
+      for (uint32_t i = 0; i < kMaxPhases - 1; ++i) mbar_init(&go[i], 1);
+      mbar_init(&drained[0], 1);
+      mbar_init(&drained[1], 1);
+      s_abort = 0;
+      fence_barrier_init();
     }
-    mbar_init(&xch_full, 1);
-    mbar_init(&xch_free, 1);
-    for (uint32_t i = 0; i < kMaxPhases - 1; ++i) mbar_init(&go[i], 1);
-    mbar_init(&drained[0], 1);
-    mbar_init(&drained[1], 1);
-    s_abort = 0;
+  } else if (warp == 0) {
+    if (lane < n_stages) init_stage(lane);
+    if (lane < x_slots) init_x(lane);
+    if (lane < kSlots) init_acc(lane);
+    if (lane < kMaxPhases - 1) mbar_init(&go[lane], 1);
+    if (lane < 2) mbar_init(&drained[lane], 1);
+    if (lane == 0) {
+      mbar_init(&xch_full, 1);
+      mbar_init(&xch_free, 1);
+      s_abort = 0;
+    }
     fence_barrier_init();
   }
   if (warp == 2) tmem_alloc(&s_tmem, tmem_cols(kN));
@@ -494,36 +512,49 @@ __global__ void __maxnreg__(kN == 256 ? 96 : 80) gemv_pair_kernel(const __grid_c
     pdl_wait();
     // fill(kb, xs): the k blocks of slot xs, from kb on.  For every slot of a phase that this warp fills.
     auto each_slot = [&](const PairPhase& q, const Part& w, auto fill) -> bool {
-      auto put = [&](uint32_t kb, uint32_t kb_end, uint32_t first, uint32_t& at, uint32_t& par) -> bool {   // into the next slots of a pipeline
+      [[maybe_unused]] auto put = [&](uint32_t kb, uint32_t kb_end, uint32_t first) -> bool {   // into the next slots of this warp's pipeline
         for (; kb < kb_end; kb += kXB) {
-          if (!wait(empty_a + (first + at) * 8, par)) return false;
-          fill(kb, first + at);
-          if (++at == pipe_slots) { at = 0; par ^= 1u; }
+          if (!wait(empty_a + (first + stage) * 8, parity)) return false;
+          fill(kb, first + stage);
+          if (++stage == pipe_slots) { stage = 0; parity ^= 1u; }
         }
         return true;
       };
       for (uint32_t pa = w.u0; pa < w.u1; pa += w.run) {
         if constexpr (kPipes == 1) {
-          if (!put(w.kb0, w.kb1, 0, stage, parity)) return false;
+          if (!put(w.kb0, w.kb1, 0)) return false;
         } else {
           const uint32_t chunk = chunk_blocks(kN, q.image), slot_n = q.slot_blocks, in_turn = slots_in_turn(kN, q.image, slot_n);
           uint32_t turn = pipe;
           for (uint32_t k0 = w.kb0; k0 < w.kb1; k0 += slot_n, turn ^= in_turn) {
             const uint32_t k1 = min(k0 + slot_n, w.kb1);
-            for (uint32_t c = k0 + turn * chunk; c < k1; c += 2 * chunk) {
-              if constexpr (kXB == 2) {   // a chunk is a slot
-                if (!wait(empty_a + stage * 8, parity)) return false;
-                fill(c, stage);
-                if (++stage == pipe_slots) { stage = 0; parity ^= 1u; }
-                if (c + 2 < k1) {
-                  if (!wait(empty_a + (pipe_slots + stage1) * 8, parity1)) return false;
-                  fill(c + 2, pipe_slots + stage1);
-                  if (++stage1 == pipe_slots) { stage1 = 0; parity1 ^= 1u; }
+            if constexpr (kXB == 2) {   // a chunk is a slot, and this warp fills both pipelines'
+              static_assert(chunk_blocks(kN, 8) == 2 && chunk_blocks(kN, 16) == 2 && x_warps(kN) == 1);
+              if constexpr (kN == 32) {   // (6-layer 8B step of 32 sequences 979 us, with the loop below 987; small models of up to 16: that 0.3 - 1 % faster)
+                for (uint32_t c = k0; c < k1; c += 4) {
+                  if (!wait(empty_a + stage * 8, parity)) return false;
+                  fill(c, stage);
+                  if (++stage == pipe_slots) { stage = 0; parity ^= 1u; }
+                  if (c + 2 < k1) {
+                    if (!wait(empty_a + (pipe_slots + stage1) * 8, parity1)) return false;
+                    fill(c + 2, pipe_slots + stage1);
+                    if (++stage1 == pipe_slots) { stage1 = 0; parity1 ^= 1u; }
+                  }
                 }
               } else {
-              if (!put(c, min(c + chunk, k1), pipe * pipe_slots, stage, parity)) return false;
-              if (x_warps(kN) == 1 && !put(c + chunk, min(c + 2 * chunk, k1), pipe_slots, stage1, parity1)) return false;
+                for (uint32_t c = k0; c < k1; c += 2) {
+                  const bool second = ((c - k0) & 2u) != 0;
+                  const uint32_t at = second ? stage1 : stage, slot = at + (second ? pipe_slots : 0u);
+                  if (!wait(empty_a + slot * 8, second ? parity1 : parity)) return false;
+                  fill(c, slot);
+                  const bool wrap = at + 1 == pipe_slots;
+                  if (second) { stage1 = wrap ? 0u : at + 1; parity1 ^= wrap; } else { stage = wrap ? 0u : at + 1; parity ^= wrap; }
+                }
               }
+            } else {
+              static_assert(x_warps(kN) == 2);
+              for (uint32_t c = k0 + turn * chunk; c < k1; c += 2 * chunk)
+                if (!put(c, min(c + chunk, k1), pipe * pipe_slots)) return false;
             }
           }
         }
