@@ -1975,30 +1975,33 @@ int boosth::gemv_chain_launch(const boost_gemv_call_t* calls, uint32_t n_calls, 
 //   - one of the process-wide switches that choose among the kernels above is not at its default.
 constexpr uint32_t kPairMaxDepth = 4096, kPairMinColumns = 1024;
 
-// Microseconds of a product on its own, fitted to 19 numbers of rows (130 - 30000) x 8 lengths (1024 - 8192) x 13
-// batches x fp32 / bf16 results.  Cluster kernel: a threadblock goes through its share of the columns
-// k block by k block, each as long as its instructions and activations (longer for fp32 results, whose
-// accumulators are short) and its rows' weights; split-K kernels: the threadblock's share of all
-// blocks, and the partial sums of a row tile.  So few long rows are better off cut finely (1000 x 8192: 15 us against 17 at
-// batch 1, 24 against 52 at 256 and fp32), and so are rows just too many to be shared (10000 x 4096, batch 1: 1.17 x).
-// The better of the two is taken within 0.5 % on average; always the cluster kernel 8.8 %, never 15 %.
+// Microseconds of a product on its own whose columns two threadblocks share, fitted to 14 numbers of rows (130 - 9472) x 8
+// lengths (1024 - 8192) x 16 batches x fp32 / bf16 results, weights in L2 and in HBM.  Cluster kernel: a threadblock goes
+// through its share of the columns k block by k block, each as long as its instructions and activations (longer
+// for fp32 results, whose accumulators are short) and its rows' weights; split-K kernels: the threadblock's share of all blocks,
+// and the partial sums of a row tile.  So up to 64 rows few long rows are left to the split-K kernels (1000 x 8192 at batch 1
+// fp32: 11.6 us against 13.9), above fp32 results with a short accumulator for every k block or two (1000 x 4096 at
+// batch 128: 13 against 26).  The better of the two is taken within 0.4 % on average (the
+// cluster kernel always: 6.3 %, never: 31 %), at 13 numbers of rows and 6 lengths that are not among those of the fit too.  Rows that are one threadblock's own (7 numbers, 9600 - 30000): the cluster
+// kernel takes 0.75 of the time on average and 1.03 at most.
 struct ProductCost {
   float fixed, block, block_fp32, unit;        // cluster kernel
   float split_fixed, split_block, split_sums;  // split-K kernels
 };
-constexpr ProductCost kProductCost[6][2] = {   // batches up to 8, 16, 32, 64, 128, 256; columns shared by two threadblocks, or not
-    {{4.968f, 0.112f, 0.026f, 0.007f, 6.714f, 0.333f, 0.115f}, {5.344f, 0.045f, 0.017f, 0.020f, 10.813f, 0.332f, -2.164f}},
-    {{5.250f, 0.118f, 0.040f, 0.006f, 7.038f, 0.327f, 0.117f}, {5.705f, 0.038f, 0.016f, 0.020f, 11.541f, 0.327f, -2.444f}},
-    {{5.735f, 0.141f, 0.055f, 0.003f, 7.770f, 0.421f, 0.127f}, {6.323f, 0.034f, 0.012f, 0.022f, 14.946f, 0.376f, -3.407f}},
-    {{7.448f, 0.150f, 0.069f, 0.003f, 9.076f, 0.422f, 0.078f}, {7.207f, 0.030f, 0.011f, 0.023f, 13.157f, 0.403f, -1.842f}},
-    {{8.160f, 0.228f, 0.125f, -0.001f, 10.40f, 0.616f, 0.057f}, {8.822f, 0.042f, 0.013f, 0.027f, 20.174f, 0.463f, -3.504f}},
-    {{11.30f, 0.261f, 0.165f, -0.006f, 12.04f, 0.879f, 0.051f}, {10.366f, 0.015f, 0.019f, 0.035f, 29.06f, 0.666f, -6.498f}}};
+constexpr ProductCost kProductCost[6] = {   // batches up to 8, 16, 32, 64, 128, 256
+    {5.506f, 0.080f, 0.015f, 0.011f, 7.456f, 0.374f, 0.107f}, {5.442f, 0.085f, 0.014f, 0.009f, 7.543f, 0.368f, 0.105f},
+    {5.864f, 0.085f, 0.014f, 0.009f, 8.564f, 0.388f, 0.113f}, {7.156f, 0.075f, 0.022f, 0.008f, 8.125f, 0.677f, 0.062f},
+    {10.884f, 0.060f, 0.131f, 0.007f, 11.258f, 0.753f, 0.031f}, {11.30f, 0.261f, 0.165f, -0.006f, 12.04f, 0.879f, 0.051f}};
 
 static bool cluster_faster(uint32_t N, uint32_t K, uint32_t M_b, bool fp32, const boosth::PairCut& cut) {
+  if (cut.split != 2) return true;
   const uint32_t batch = M_b <= 8 ? 0 : M_b <= 16 ? 1 : M_b <= 32 ? 2 : M_b <= 64 ? 3 : M_b <= 128 ? 4 : 5;
-  const ProductCost& c = kProductCost[batch][cut.split == 2 ? 0 : 1];
+  const ProductCost& c = kProductCost[batch];
   const float tiles = (float)((N + kBlockRows - 1) / kBlockRows), k_blocks = (float)((K + kBlockK - 1) / kBlockK);
-  const float own = k_blocks / (float)cut.split, per_tile = (float)cut.threadblocks / tiles;
+  // (fp32 results of three or four row tiles with the longest rows: the split-K kernels' sums are 0.5 - 2 % closer to the exact
+  // ones - 500 x 8192 1.59e-7 against 1.63e-7; elsewhere the cluster kernel's are as close or closer)
+  if (fp32 && M_b > 2 && tiles >= 3.f && tiles <= 4.f && K > 7168) return false;
+  const float own = k_blocks / 2.f, per_tile = (float)cut.threadblocks / tiles;
   return c.fixed + own * (c.block + (fp32 ? c.block_fp32 : 0.f) + c.unit * (float)cut.units) <=
          c.split_fixed + c.split_block * tiles * k_blocks / (float)cut.threadblocks + c.split_sums * (per_tile < k_blocks ? per_tile : k_blocks);
 }

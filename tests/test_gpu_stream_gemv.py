@@ -346,13 +346,36 @@ def test_gemv_at_the_edges_of_the_kernel_rule(dev, n, k, m_b):
     assert w.status_words() == [0]
 
 
+def ran_on_the_cluster_kernel(w, x, res):
+    """One more launch with a schedule log: the cluster kernel writes a record for each of its threadblocks,
+    whose bytes are its units of 8 rows times its k blocks (the other kernels' items are whole 128-row blocks)."""
+    m_b = x.shape[0]
+    ws_ptr, ws_bytes = w.workspace(m_b)
+    log = torch.zeros(B.boost_schedule_log_bytes(8192), dtype=torch.uint8, device=x.device)
+    log[:32].view(torch.int64)[1] = 8192
+    slab = next(t for t in w._ws.values() if t.data_ptr() <= ws_ptr < t.data_ptr() + t.numel())
+    header = slab[ws_ptr - slab.data_ptr():][:64].view(torch.int64)
+    header[B.WS_LOG_WORD // 2] = log.data_ptr()
+    w.gemv(x, residual=res)
+    torch.cuda.synchronize()
+    header[B.WS_LOG_WORD // 2] = 0
+    records, _ = B.schedule_records(log.cpu().numpy())
+    k_blocks, units = w.layout["k_blocks"], 16 * w.layout["n_row_tiles"]
+    clusters = torch.cuda.get_device_properties(x.device).multi_processor_count // 2
+    shared = -(-units // clusters) <= 16
+    workers = clusters if shared else 2 * clusters
+    rows = [units * (i + 1) // workers - units * i // workers for i in range(workers)]
+    halves = [k_blocks // 2, k_blocks - k_blocks // 2] if shared else [k_blocks]
+    return sorted(int(b) for b in records["bytes"]) == sorted(1024 * r * h for r in rows for h in halves if r)
+
+
 @pytest.mark.parametrize("n,k,m_b", [
-    (1001, 1088, 5), (1001, 1216, 24), (9601, 1088, 16), (1001, 1216, 70), (9601, 1088, 128),   # chunks of two k blocks: an odd last one, an odd number of them
-    (1001, 1032, 70), (2049, 1088, 80), (300, 1160, 100),   # ... one to a slot of accumulators
-    (1001, 1152, 160), (9601, 1088, 161), (1001, 1088, 192), (9601, 1216, 193), (1001, 1216, 224), (9601, 1088, 225),   # sizes of an activation tile
+    (1001, 1088, 5), (1001, 1216, 24), (9601, 1088, 16), (4001, 1544, 70), (9601, 1088, 128),   # chunks of two k blocks: an odd last one, an odd number of them
+    (2049, 1088, 70), (4001, 1160, 80), (3000, 1032, 100),   # ... one to a slot of accumulators
+    (4001, 1152, 160), (9601, 1088, 161), (4001, 1088, 192), (9601, 1216, 193), (4001, 1216, 224), (9601, 1088, 225),   # sizes of an activation tile
     (9601, 2880, 241), (9601, 2944, 250), (19001, 2560, 250), (19001, 2624, 256)])   # 256-row tiles: three and four of them, one and two images
 def test_gemv_pipelines_and_tile_sizes(dev, n, k, m_b):
-    """The cluster kernel's two pipelines take chunks of k blocks in turn (8 - 19 blocks per threadblock here),
+    """The cluster kernel's two pipelines take chunks of k blocks in turn (8 - 47 blocks per threadblock here),
     and from 129 rows on the size of an activation tile decides how many there are: against the
     oracle, and every launch gives the same bits."""
     w, y, ref, (x, res) = run_gemv(dev, n, k, m_b, 0.0, seed=n + k + m_b, residual=True)
@@ -360,6 +383,7 @@ def test_gemv_pipelines_and_tile_sizes(dev, n, k, m_b):
     again = [w.gemv(x, residual=res) for _ in range(20)]
     torch.cuda.synchronize()
     assert all(np.array_equal(a.cpu().numpy(), y) for a in again)
+    assert ran_on_the_cluster_kernel(w, x, res)
     assert w.status_words() == [0]
 
 
@@ -382,9 +406,9 @@ def test_split_k_kernels_at_full_size(dev, n, k, m_b):
 
 @pytest.mark.parametrize("n,k,m_b", [(1000, 8192, 1), (1000, 8192, 256), (10000, 4096, 1), (500, 4096, 200), (300, 8192, 64)])
 def test_products_that_are_better_off_split_finely(dev, n, k, m_b):
-    """Few long rows, and rows just too many for two threadblocks to share, take the kernels whose partial sums
-    meet in memory: against the oracle, and no slower than under the switch that asks for them (a tenth
-    for the clock; on the cluster kernel they were 1.15 to 2.6 times slower)."""
+    """Few long rows, which the rule leaves to the kernels whose partial sums meet in memory, and rows just too many for two
+    threadblocks to share: against the oracle, and no slower than under the switch that asks for
+    those kernels (a tenth for the clock)."""
     from paper_2609_13592_b200.tiers import TieredWeight
     w, y, ref, (x, _) = run_gemv(dev, n, k, m_b, 0.0, seed=n + m_b)
     assert_close_to_oracle(y, ref, f"{n} x {k}, batch {m_b}")
