@@ -313,10 +313,10 @@ __device__ __noinline__ uint32_t host_bytes_of_range(const PairPhase& q, uint32_
   return bytes;
 }
 
-// Registers: beside an attention threadblock (up to 32 rows) and within an SM (up to 128) as many as measured best: hidden
-// 256, 24 sequences with 80 77.1 us, with 96 75.8; 12 sequences with 80 66.1, with 88 65.1; 8B steps the same.
+// Registers: beside an attention threadblock (up to 32 rows) and within an SM (64, 128) as many as measured best (32 rows: 80 / 88,
+// hidden 256, 18 - 30 sequences of 20 - 100 tokens 1.015 / 1.002 of the time before the second pipeline).
 template <uint32_t kN, uint32_t kChunk>
-__global__ void __maxnreg__(kN >= 256 || kN == 32 ? 96 : kN == 16 ? 88 : 80) gemv_pair_kernel(const __grid_constant__ PairParams p) {
+__global__ void __maxnreg__(kN >= 256 ? 96 : kN == 32 ? 88 : 80) gemv_pair_kernel(const __grid_constant__ PairParams p) {
   constexpr uint32_t kXB = x_blocks(kN), kSlots = acc_slots(kN), kSlotCols = slot_cols(kN), kPipes = pipes_of(kN);
   constexpr bool kTmaX = x_by_tma(kN);
   constexpr uint32_t kEpiWarps = epi_warps(kN), kEpiThreads = kEpiWarps * 32;
@@ -1359,21 +1359,28 @@ uint32_t clusters_for(uint32_t M_b) {
 // average number of blocks of 8 rows x 64 columns in an image.  Products on their own (9600 - 60000 rows x 1024 - 4096
 // columns): the times meet at 330 - 430 blocks for fp32 results, 390 - 460 for bf16, the lower ones where there is another
 // image, whose MMAs hide the epilogue (28672 x 1024, 194 blocks: 32 columns 30.6 us, 64 27.7; 14336 x 4096, 775: 41.5, 45.1).
-// Chains of a step: six models of 300 - 470 blocks 0 - 2 % faster with 64, one of 775 (the 8B model) 4 % with 32.
+// Steps: six models of 300 - 540 blocks 0 - 2 % faster with 64, one of 775 (the 8B model) 4 % with 32.
+// Where all rows of a step's launch are shared and its K is short, 64 (hidden 256 / 512, batch 200 - 240: 1.8 / 0.5 % faster); a
+// step's first launch, a product on its own, is counted as one too: two forms of the kernel in turn cost 2 us a step.
 bool wide_chunk(const PairParams& p) {
-  if (p.nb <= 224) return p.nb <= 192;
+  if (p.nb <= 192) return true;
   const uint32_t clusters = clusters_for(p.M_b);
-  bool wide = false;
+  const bool step = p.early || p.n_phases > 1;
+  bool own_rows = false, shared_short = step;
   for (uint32_t i = 0; i < p.n_phases; ++i) {
     PairPhase q = p.ph[i];
     plan_phase(q, clusters, 256, p.M_b);
-    if (q.split == 2) continue;
+    if (q.split == 2) {
+      shared_short = shared_short && q.k_blocks <= 32;
+      continue;
+    }
+    if (p.nb < 256) return false;
     const bool fp32 = q.epi == BOOST_EPI_PLAIN && q.y_dtype == 0;
-    const uint32_t most = p.n_phases > 1 ? 500u : q.max_images > 1 ? (fp32 ? 330u : 390u) : fp32 ? 372u : 440u;
+    const uint32_t most = step ? 600u : q.max_images > 1 ? (fp32 ? 330u : 390u) : fp32 ? 372u : 440u;
     if ((uint64_t)q.n_units * q.k_blocks > (uint64_t)most * 2 * clusters * q.max_images) return false;
-    wide = true;
+    own_rows = true;
   }
-  return wide;
+  return own_rows || shared_short;
 }
 
 // Row statistics between the phases of one launch live in two buffers of the workspace; a phase's
