@@ -37,7 +37,7 @@ FALLBACK_HBM_GBS = 6650.0
 # DRAM bytes (read + write) per algorithmic byte of the weight products of a 32-layer step, from ncu
 # captures of this workload's launches at batch 32 and 128
 GEMV_TRAFFIC_PROFILE = "profiles/gemv_pair_kernel_llama8b.md"
-GEMV_TRAFFIC = {32: 1.014, 128: 1.036}
+GEMV_TRAFFIC = {32: 1.013, 128: 1.035}
 
 
 def load_peaks():
@@ -564,8 +564,9 @@ def run_ours(args, rank, world, local_rank):
                          "achieved": gemv_gbs, "peak": hbm_peak, "unit": "GB/s", "frac": gemv_gbs / hbm_peak,
                          "algorithmic_bytes_per_launch": gemv_bytes_per_launch,
                          "traffic": GEMV_TRAFFIC[32 if batch <= 32 else 128] * gemv_bytes_per_launch,
-                         "traffic_source": ("ncu dram bytes of this workload's launches, ratio 1.014 to algorithmic" if batch <= 32 else
-                                            "ncu dram bytes of the same launches at batch 128, ratio 1.036 to algorithmic"),
+                         "traffic_source": ("ncu dram bytes of this workload's launches (two layers of them)" if batch <= 32 else
+                                            "ncu dram bytes of the same launches at batch 128 (two layers of them)") +
+                                           f", ratio {GEMV_TRAFFIC[32 if batch <= 32 else 128]} to algorithmic",
                          "launches_per_step": gemv_n, "avg_launch_us": 1e3 * gemv_ms / max(gemv_n, 1),
                          "peak_source": peak_src,
                          # events around every launch serialise the step: no launch overlaps its neighbours

@@ -1978,12 +1978,14 @@ constexpr uint32_t kPairMaxDepth = 4096, kPairMinColumns = 1024;
 // Microseconds of a product on its own whose columns two threadblocks share, fitted to 14 numbers of rows (130 - 9472) x 8
 // lengths (1024 - 8192) x 16 batches x fp32 / bf16 results, weights in L2 and in HBM.  Cluster kernel: a threadblock goes
 // through its share of the columns k block by k block, each as long as its instructions and activations (longer
-// for fp32 results, whose accumulators are short) and its rows' weights; split-K kernels: the threadblock's share of all blocks,
-// and the partial sums of a row tile.  So up to 64 rows few long rows are left to the split-K kernels (1000 x 8192 at batch 1
-// fp32: 11.6 us against 13.9), above fp32 results with a short accumulator for every k block or two (1000 x 4096 at
-// batch 128: 13 against 26).  The better of the two is taken within 0.4 % on average (the
-// cluster kernel always: 6.3 %, never: 31 %), at 13 numbers of rows and 6 lengths that are not among those of the fit too.  Rows that are one threadblock's own (7 numbers, 9600 - 30000): the cluster
-// kernel takes 0.75 of the time on average and 1.03 at most.
+// for fp32 results, whose accumulators are short) and its rows' weights; split-K kernels: the threadblock's share of
+// all blocks, and the partial sums of a row tile.  So up to 64 rows few long rows are left to the split-K kernels (1000 x
+// 8192 at batch 1, fp32 results: 11.6 us against 13.6), above fp32 results with an accumulator for every k block or two
+// (1000 x 4096 at batch 128: 13.0 against 25.8).  The better of the two is taken within 0.4 % on average (the cluster
+// kernel always: 6.3 %, never: 31 %), at 13 numbers of rows and 6 lengths that are not among those of the fit too.  The
+// last row is of an earlier fit (within 0.8 %: a new one moved few products, half of them the wrong way).
+// Rows that are one threadblock's own (7 numbers, 9600 - 30000): the cluster kernel takes 0.75 of the time on
+// average and 1.03 at most.
 struct ProductCost {
   float fixed, block, block_fp32, unit;        // cluster kernel
   float split_fixed, split_block, split_sums;  // split-K kernels

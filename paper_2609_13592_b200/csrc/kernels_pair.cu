@@ -23,8 +23,8 @@
 // activation tiles side by side took fewer MMAs and the same time, but half of its results were
 // nobody's: at batch 32 the GPU is at its power limit, and a step of 4690 us became one of 4640.)
 //
-// One threadblock per SM.  Up to 32 batch rows it takes 147 KiB of shared memory and 80 registers per
-// thread: a threadblock of the attention kernel before and after it on the stream fits beside it, and
+// One threadblock per SM.  Up to 32 batch rows it takes 147 KiB of shared memory and 88 registers per
+// thread at most: a threadblock of the attention kernel before and after it on the stream fits beside it, and
 // the weights of the first product are in place when the kernel before it ends.  A ring of 64 KiB
 // per SM already saturates HBM (measured with bulk copies of 2 - 16 KiB: 48 KiB 6.3, 64 KiB 6.8, 80
 // - 112 KiB 6.9, 192 KiB 6.4 - 6.7 TB/s), so sharing the SM costs no bandwidth.  Larger batches take
@@ -33,7 +33,8 @@
 // Warps: 0 and 3 weight producers (a pipeline each, or every other stage: one warp's instruction latency
 // would bound the stream of a product whose stages are four or eight copies), 1 activation producer, 2 MMA
 // issue and tensor-memory allocation, 4 and up epilogue, behind them (up to 128 rows) the second
-// pipeline's MMA issue and (128 rows) activation producer.  Producers and MMA warps run warp-uniform code and elect a lane for the copy or MMA itself: inside an if (lane == 0) every operand goes through a
+// pipeline's MMA issue and (128 rows) activation producer.  Producers and MMA warps run warp-uniform code
+// and elect a lane for the copy or MMA itself: inside an if (lane == 0) every operand goes through a
 // vector register (measured: a group of four MMAs and a commit 293 cycles against 212, a bulk copy 64
 // against 25).
 #include <cuda.h>
@@ -1352,9 +1353,9 @@ uint32_t clusters_for(uint32_t M_b) {
 }
 
 // 129 - 256 rows: 64 columns to an epilogue's chunk, or 32?  Where four activation slots fit beside 64 that is better (tiles of
-// up to 192 rows: 6-layer step at batch 180 1518 us, with 32 and a stage more 1540).  Tiles of 224 rows: 32, and
-// a fourth slot in the room that leaves (batch 200: 1767 -> 1615).  Of 256 rows: the fourth slot pays where a product waits
-// for activations (batch 250: 1907 -> 1820), and 64 columns, with three slots, where rows that are one threadblock's
+// up to 192 rows: 6-layer step at batch 180 1511 us, with 32 and a stage more 1523).  Tiles of 224 rows: 32, and
+// a fourth slot in the room that leaves (batch 200: 1763 -> 1610).  Of 256 rows: the fourth slot pays where a product waits
+// for activations (batch 250: 1903 -> 1820), and 64 columns, with three slots, where rows that are one threadblock's
 // have few k blocks, so that the epilogue is most of its time.  Measured at batch 232 - 256, weights from HBM, by the
 // average number of blocks of 8 rows x 64 columns in an image.  Products on their own (9600 - 60000 rows x 1024 - 4096
 // columns): the times meet at 330 - 430 blocks for fp32 results, 390 - 460 for bf16, the lower ones where there is another
@@ -1393,7 +1394,7 @@ int launch_pair(PairParams& p, float* stats, size_t stats_bytes, cudaStream_t st
   if (clusters == 0) return BOOST_ERR_UNSUPPORTED;
   // activation slots: more than a microsecond of a short product's stream (a k block per 155 ns); from
   // 128 rows on half of the shared memory and more, since the tiles are as large as the weight stages.  Above 128 rows
-  // four tiles, five where that leaves five stages (batch 150: 1431 -> 1388 us for 6 layers; 180: four 1518, five 1550), and
+  // four tiles, five where that leaves five stages (batch 150: 1424 -> 1384 us for 6 layers; 180: four 1511, five 1652), and
   // of 256 rows three where the chunks have 64 columns.
   const uint32_t slot_bytes = x_blocks(kN) * p.nb * 128u;
   const uint32_t x_budget = kN <= 16 ? 6 * slot_bytes : kN == 32 ? 4 * slot_bytes : kN == 64 ? 64u * 1024u : kN == 128 ? 96u * 1024u : (p.nb <= 160 ? 5 : p.nb == 256 && kChunk == 64 ? 3 : 4) * slot_bytes;
